@@ -69,9 +69,7 @@ int fail(int code, const std::string &msg) {
             return fail(CAMP_E_CUDA, std::string(#x) + ": " + cudaGetErrorString(e_)); \
     } while (0)
 
-// dynamic shared memory one block may use (227 KB less room for a block
-// group's static reduction scratch)
-const int kMaxSmem = 227 * 1024 - 256;
+const int kMaxSmem = CAMP_MAX_SMEM;
 
 int check_device(const camp_mech *m) {
     if (!m->on_device) return fail(CAMP_E_INVAL, "mechanism was compiled without device tables");
@@ -111,7 +109,7 @@ int camp_pick_shape(int n, int lanes) {
 }
 
 int camp_cell_smem_bytes(const DevMech &m, int lu_elem) {
-    return campdev::cell_smem(m.n, m.R, m.n_rev, m.nlu, lu_elem, m.n_part, m.n_pw, m.n_pw64).bytes;
+    return (lu_elem == 4 ? m.smem4 : m.smem8).bytes;
 }
 
 cudaError_t camp_launch_rates(const DevMech &m, long long n_cells, const double *env, double *kf,

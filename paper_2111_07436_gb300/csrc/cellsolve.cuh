@@ -40,53 +40,33 @@ constexpr double NAV = 6.02214076e23;
 constexpr double RG = KB * NAV;
 constexpr double PI_D = 3.14159265358979323846;
 
-// ---- shared-memory layout of one cell --------------------------------------
-struct CellSmem {
-    int ys, rs, kf, kr, pw, x, lu, bytes;
-};
-__host__ __device__ inline int align16(int b) { return (b + 15) & ~15; }
-// rs holds the R rate terms, then n_part partial sums (of split forcing sums
-// inside an f evaluation, of split substitution rows inside a solve)
-// pw holds the water parameter's per-cell values (n_pw doubles, and n_pw64
-// more in the FP64 form; none without one)
-__host__ __device__ inline CellSmem cell_smem(int n, int R, int n_rev, int nlu, int lu_elem, int n_part,
-                                              int n_pw, int n_pw64) {
-    CellSmem c;
-    int o = 0;
-    c.ys = o; o = align16(o + 8 * n);
-    c.rs = o; o = align16(o + 8 * (R + n_part));
-    c.kf = o; o = align16(o + 8 * R);
-    c.kr = o; o = align16(o + 8 * n_rev);
-    c.pw = o; o = align16(o + 8 * (n_pw + (lu_elem == 8 ? n_pw64 : 0)));
-    // the substitution vector shares the rate-term scratch when it fits:
-    // the rate terms live only inside one f evaluation, the vector only
-    // inside one Newton solve, and the Jacobian assembly keeps its FP32
-    // copy of y in ys instead
-    if (8 * R >= lu_elem * n) {
-        c.x = c.rs;
-    } else {
-        c.x = o;
-        o = align16(o + lu_elem * n);
-    }
-    c.lu = o; o = align16(o + lu_elem * nlu);
-    c.bytes = o;
-    return c;
-}
-
+// ---- one cell's shared memory (cell_smem) -----------------------------------
+// The arrays of one cell in the block's dynamic shared memory, from the cell's
+// byte offset in it.  The layout comes precomputed with the mechanism (in the
+// constant bank), and every pointer is visibly one into shared memory, also
+// in the functions kept out of line.
+extern __shared__ __align__(16) char block_smem[];
 template <typename LT>
 struct CellPtr {
-    double *ys, *rs, *kf, *kr, *pw;
+    double *ys, *rs, *kf, *kr, *pw, *fb;
     LT *x, *lu;
-    __device__ CellPtr(char *base, const DevMech &m) {
-        CellSmem c = cell_smem(m.n, m.R, m.n_rev, m.nlu, (int)sizeof(LT), m.n_part, m.n_pw, m.n_pw64);
-        ys = (double *)(base + c.ys);
-        rs = (double *)(base + c.rs);
-        kf = (double *)(base + c.kf);
-        kr = (double *)(base + c.kr);
-        pw = (double *)(base + c.pw);
-        x = (LT *)(base + c.x);
-        lu = (LT *)(base + c.lu);
+    int base;
+    __device__ __forceinline__ CellPtr(int b, const DevMech &m) : base(b) {
+        const CellSmem &c = layout(m);
+        ys = (double *)(block_smem + b + c.ys);
+        rs = (double *)(block_smem + b + c.rs);
+        kf = (double *)(block_smem + b + c.kf);
+        kr = (double *)(block_smem + b + c.kr);
+        pw = (double *)(block_smem + b + c.pw);
+        x = (LT *)(block_smem + b + c.x);
+        lu = (LT *)(block_smem + b + c.lu);
+        fb = (double *)(block_smem + b + c.fb);
     }
+    static __device__ __forceinline__ const CellSmem &layout(const DevMech &m) {
+        return sizeof(LT) == 4 ? m.smem4 : m.smem8;
+    }
+    // whether the odd halves of the forcing sums have their own array (fb)
+    static __device__ __forceinline__ bool halves(const DevMech &m) { return layout(m).fb >= 0; }
 };
 
 // ---- group primitives --------------------------------------------------------
@@ -165,7 +145,7 @@ __device__ __forceinline__ double section_volume(const DevMech &m, const double 
 // Rate constants of process k: env holds T, P and the runtime rates; sec the
 // (radius, number concentration, liquid volume) of the section (or particle)
 // a section process acts in (unused by the others)
-__device__ inline void rate_constant_at(const DevMech &m, int k, const double *__restrict__ env,
+static __device__ __noinline__ void rate_constant_at(const DevMech &m, int k, const double *__restrict__ env,
                                         const double *__restrict__ sec, double &kf, double &kr) {
     const double T = env[0], P = env[1];
     const double Mair = P / (KB * T) * 1e-6;  // molec cm^-3
@@ -270,20 +250,72 @@ __device__ __forceinline__ void rate_constant(const DevMech &m, int k, const dou
     rate_constant_at(m, k, env, sec, kf, kr);
 }
 
+// ---- FP64 without the FP64 pipe -----------------------------------------------
+// Every FP64 instruction of a warp -- conversions between FP32 and FP64 and
+// FP64 comparisons included -- holds its SM sub-partition's FP64 port for 64
+// cycles, however many lanes are active and however independent it is of the
+// others (measured: 64 cycles an instruction for one warp at any ILP, one per
+// 16-19 cycles over a whole SM).  The integer pipe issues tens of instructions
+// in that time, so the conversions and comparisons of the solve's inner loops
+// run there, with the same results bit for bit.
+
+// (float)x, rounded to nearest even.  In range (an FP32 normal result): the
+// exponent is re-biased and the 29 dropped bits rounded in by an integer
+// carry.  Zeros and values below half the smallest FP32 denormal are signed
+// zeros; FP32 denormals, overflows, infinities and NaN take the conversion
+// instruction.
+__device__ __forceinline__ float narrow(double x) {
+    const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
+    const unsigned ex = (hi >> 20) & 0x7ffu, sign = hi & 0x80000000u;
+    unsigned u = __funnelshift_l(lo, hi, 3) + 0x40000000u;  // (ex - 896) << 23 | top 23 fraction bits
+    u += ((lo & 0x1fffffffu) + 0x0fffffffu + (u & 1u)) >> 29;
+    if (ex - 897u >= 254u) {
+        if (ex < 873u) u = 0u;
+        else return (float)x;
+    }
+    return __uint_as_float(u | sign);
+}
+// (double)x, exact: normal values and zeros by shifts, the rest by the
+// conversion instruction
+__device__ __forceinline__ double widen(float x) {
+    const unsigned b = __float_as_uint(x), a = b & 0x7fffffffu, sign = b & 0x80000000u;
+    if (a - 0x00800000u >= 0x7f000000u) {
+        if (a == 0u) return __hiloint2double((int)sign, 0);
+        return (double)x;
+    }
+    return __hiloint2double((int)(((a >> 3) + 0x38000000u) | sign), (int)(b << 29));
+}
+// a > b and a >= b for b >= +0 and any a (false for a NaN or negative a, as
+// the FP64 comparisons are; a = -0 compares below +0 here, which no caller
+// can pass)
+constexpr long long INF_BITS = 0x7ff0000000000000ll;
+__device__ __forceinline__ bool pos_gt(double a, double b) {
+    const long long x = __double_as_longlong(a);
+    return x > __double_as_longlong(b) && x <= INF_BITS;
+}
+__device__ __forceinline__ bool pos_ge(double a, double b) {
+    const long long x = __double_as_longlong(a);
+    return x >= __double_as_longlong(b) && x <= INF_BITS;
+}
+
 // FP64 values into and out of the LU precision
 template <typename LT> __device__ __forceinline__ LT to_lu(double x);
-template <> __device__ __forceinline__ float to_lu<float>(double x) { return (float)x; }
+template <> __device__ __forceinline__ float to_lu<float>(double x) { return narrow(x); }
 template <> __device__ __forceinline__ double to_lu<double>(double x) { return x; }
-__device__ __forceinline__ double from_lu(float x) { return (double)x; }
+__device__ __forceinline__ double from_lu(float x) { return widen(x); }
 __device__ __forceinline__ double from_lu(double x) { return x; }
 
 // One lane's term (x w)^2 of the Newton update's squared norm, in the LU
 // precision.  In FP32 a weight beyond the format's range (atol below ~3e-39
 // on a species near zero) is held at its largest value and the product at
 // 1e18, so the sum stays finite; either only arises far from convergence.
-// A non-finite x is caught separately.
-__device__ __forceinline__ float upd_term(float x, double w) {
-    const float t = fminf(fabsf(x * fminf((float)w, 3.4e38f)), 1e18f);
+// A non-finite x is caught separately.  norm_weight: the weight as the norm
+// takes it, in the LU precision (once per step).
+template <typename LT> __device__ __forceinline__ LT norm_weight(double w);
+template <> __device__ __forceinline__ float norm_weight<float>(double w) { return fminf(narrow(w), 3.4e38f); }
+template <> __device__ __forceinline__ double norm_weight<double>(double w) { return w; }
+__device__ __forceinline__ float upd_term(float x, float w) {
+    const float t = fminf(fabsf(x * w), 1e18f);
     return t * t;
 }
 __device__ __forceinline__ double upd_term(double x, double w) {
@@ -303,28 +335,89 @@ __device__ __forceinline__ int lo16(int v) { return v & 0xffff; }
 __device__ __forceinline__ int hi16(int v) { return (int)((unsigned)v >> 16); }
 constexpr int NONE16 = 0xffff;
 
-__device__ __forceinline__ double rate_term(const DevMech &m, int k, const double *ys, double kf,
-                                            const double *kr) {
-    const int4 rp = __ldg(m.rpack + k);
-    const int a0 = lo16(rp.x), a1 = hi16(rp.x), a2 = lo16(rp.y), rv = hi16(rp.y);
-    double a = kf;
-    if (a0 != NONE16) a *= ys[a0];
-    if (a1 != NONE16) a *= ys[a1];
-    if (a2 != NONE16) a *= ys[a2];
-    if (rv != NONE16) {
-        const int b0 = lo16(rp.z), b1 = hi16(rp.z), b2 = lo16(rp.w);
-        double b = kr[rv];
-        if (b0 != NONE16) b *= ys[b0];
-        if (b1 != NONE16) b *= ys[b1];
-        if (b2 != NONE16) b *= ys[b2];
-        a -= b;
+// r_k of every process into rs, G at a time.  The operands of the next
+// processes are fetched under the present ones' FP64 products, without
+// branches around the loads: a missing factor reads position 0 and is not
+// multiplied in, and only the rare third factors and reverse terms branch.
+template <int G>
+__device__ __forceinline__ void rate_terms(const DevMech &m, const double *ys, const double *kfs, const double *kr,
+                                           double *rs, int lane) {
+    const int R = m.R;
+    auto at = [&](int p) { return ys[p != NONE16 ? p : 0]; };
+    int k = min(lane, R - 1);
+    int4 rp = __ldg(m.rpack + k);
+    int4 rn = __ldg(m.rpack + min(lane + G, R - 1));
+    double a = kfs[k], y0 = at(lo16(rp.x)), y1 = at(hi16(rp.x));
+#pragma unroll 1
+    for (int b = 0; b < R; b += G) {
+        const int kn = min(lane + b + G, R - 1);
+        const int4 r2 = __ldg(m.rpack + min(lane + b + 2 * G, R - 1));
+        const double an = kfs[kn], n0 = at(lo16(rn.x)), n1 = at(hi16(rn.x));
+        if (lo16(rp.x) != NONE16) a *= y0;
+        if (hi16(rp.x) != NONE16) a *= y1;
+        if (rp.y != -1) {
+            const int a2 = lo16(rp.y), rv = hi16(rp.y);
+            const int b0 = lo16(rp.z), b1 = hi16(rp.z), b2 = lo16(rp.w);
+            if (a2 != NONE16) a *= ys[a2];
+            if (rv != NONE16) {
+                double r = kr[rv];
+                const double u0 = at(b0), u1 = at(b1);
+                if (b0 != NONE16) r *= u0;
+                if (b1 != NONE16) r *= u1;
+                if (b2 != NONE16) r *= ys[b2];
+                a -= r;
+            }
+        }
+        if (lane + b < R) rs[lane + b] = a;
+        rp = rn;
+        rn = r2;
+        a = an;
+        y0 = n0;
+        y1 = n1;
     }
-    return a;
 }
 
-__device__ __forceinline__ double gather_entry(const DevMech &m, int q, const double *rs) {
-    const int g = __ldg(m.fpk + q);
-    return __ldg(m.fcoef + hi16(g)) * rs[lo16(g)];
+// The gather of f from the rate terms: each lane runs through its flat list
+// of entry pairs (DevMech::gth), with the records two steps and the operands
+// one step ahead, so that a step costs its two FP64 products-and-sums alone.
+// A finished sum's two halves go to shared memory (ys or the partials, and
+// fb), where the owners add them: one FP64 add per position slot instead of
+// one in every step in which some lane finishes a sum.
+template <int G, bool FB>
+__device__ __forceinline__ void gather_terms(const DevMech &m, const double *rs, double *ys, double *fp, double *fb,
+                                             int lane) {
+    const int n = m.n, S = m.n_gstep;
+    const int2 *rec = m.gth + lane;
+    const double2 *cf = m.gcf + lane;
+    int2 r0 = __ldg(rec), r1 = __ldg(rec + G);
+    double2 c0 = __ldg(cf);
+    rec += 2 * G;
+    cf += G;
+    double v0 = rs[r0.x & 0x7fff], v1 = rs[hi16(r0.x) & 0x7fff];
+    double acc = 0.0, acc2 = 0.0;
+#pragma unroll 2
+    for (int s = 0; s < S; s++, rec += G, cf += G) {
+        const int2 r2 = __ldg(rec);  // two steps of padding follow the last
+        const double2 c1 = __ldg(cf);
+        const double w0 = rs[r1.x & 0x7fff], w1 = rs[hi16(r1.x) & 0x7fff];
+        if (!(r0.x & 0x8000)) acc = fma(c0.x, v0, acc);
+        if (r0.x >= 0) acc2 = fma(c0.y, v1, acc2);
+        const bool end = r0.y >= 0;
+        double *to = (G == 32 || r0.y < n) ? ys + r0.y : fp + (r0.y - n);
+        if constexpr (FB) {
+            if (end) *to = acc;
+            if (end) fb[r0.y] = acc2;
+        } else {
+            if (end) *to = acc + acc2;
+        }
+        acc = end ? 0.0 : acc;
+        acc2 = end ? 0.0 : acc2;
+        r0 = r1;
+        r1 = r2;
+        c0 = c1;
+        v0 = w0;
+        v1 = w1;
+    }
 }
 
 // ---- the water parameter (Sect. 2.2.2; Table 4, ZSRAerosolWater) ----------
@@ -405,25 +498,34 @@ __device__ __forceinline__ void water_update(const DevMech &m, double *pw, const
     gsync<G>(gm);
 }
 
+// a x^p without the products by one that ipowd's loop starts from
+__device__ __forceinline__ double times_pow(double a, double x, int p) {
+    if (p > 0) {
+        double r = x;
+        for (int i = 1; i < p; i++) r *= x;
+        a *= r;
+    }
+    return a;
+}
+
 // r_k with the powers of 1/L of a section process applied (the water build's
 // rate term)
-__device__ __forceinline__ double rate_term_water(const DevMech &m, int k, const double *ys, const double *kf,
-                                                  const double *kr, const double *invl) {
-    const int4 rp = __ldg(m.rpack + k);
+__device__ __forceinline__ double rate_term_water(const DevMech &m, int k, const int4 rp, const double *ys,
+                                                  const double *kf, const double *kr, const double *invl) {
     const WaterTag t = water_tag(rp.w);
     double il = 1.0;
     if (t.sec >= 0) {
         il = invl[t.sec];
-        if (!(il > 0.0)) return 0.0;
+        if (!pos_gt(il, 0.0)) return 0.0;
     }
     const int a0 = lo16(rp.x), a1 = hi16(rp.x), a2 = lo16(rp.y), rv = hi16(rp.y);
-    double a = kf[k] * ipowd(il, t.la);
+    double a = times_pow(kf[k], il, t.la);
     if (a0 != NONE16) a *= ys[a0];
     if (a1 != NONE16) a *= ys[a1];
     if (a2 != NONE16) a *= ys[a2];
     if (rv != NONE16) {
         const int b0 = lo16(rp.z), b1 = hi16(rp.z), b2 = lo16(rp.w);
-        double b = kr[rv] * ipowd(il, t.lb);
+        double b = times_pow(kr[rv], il, t.lb);
         if (b0 != NONE16) b *= ys[b0];
         if (b1 != NONE16) b *= ys[b1];
         if (b2 != NONE16) b *= ys[b2];
@@ -479,69 +581,70 @@ __device__ __forceinline__ void water_chain(const DevMech &m, double *pw, const 
 }
 
 // y in c.ys (written by the caller, who also made it visible to the group)
-// -> f (own positions).  The per-position sums are spread over the cell's
+// -> f in shared memory, as two halves in ys and fb (or whole in ys).  The per-position sums are spread over the cell's
 // lanes by the compiler's balanced assignment (long sums in chunks) and
-// handed back through shared memory (reusing ys).
-template <int G, int NPL, typename LT, bool W>
-__device__ __forceinline__ void eval_f_ys(const DevMech &m, const CellPtr<LT> &c, double (&f)[NPL],
-                                          int lane, unsigned gm) {
+// handed back through shared memory (reusing ys).  On return a lane may
+// write its own positions of ys and, after a group sync, anything.
+template <int G, typename LT, bool W>
+__device__ __forceinline__ void eval_f_ys(const DevMech &m, const CellPtr<LT> &c, int lane, unsigned gm) {
     if constexpr (W) {
         water_update<G>(m, c.pw, c.ys, lane, gm);
         const double *invl = pw_invl(m, c.pw);
-        for (int k = lane; k < m.R; k += G) c.rs[k] = rate_term_water(m, k, c.ys, c.kf, c.kr, invl);
+        int4 rp = __ldg(m.rpack + min(lane, m.R - 1));
+#pragma unroll 1
+        for (int k = lane; k < m.R; k += G) {
+            const int4 rn = __ldg(m.rpack + min(k + G, m.R - 1));
+            c.rs[k] = rate_term_water(m, k, rp, c.ys, c.kf, c.kr, invl);
+            rp = rn;
+        }
     } else {
-        for (int k = lane; k < m.R; k += G) c.rs[k] = rate_term(m, k, c.ys, c.kf[k], c.kr);
+        rate_terms<G>(m, c.ys, c.kf, c.kr, c.rs, lane);
     }
     gsync<G>(gm);
     double *fs = c.ys;  // y is no longer needed
     double *fp = c.rs + m.R;
-    const int b0 = __ldg(m.flane_ptr + lane), b1 = __ldg(m.flane_ptr + lane + 1);
-    for (int i = b0; i < b1; i++) {
-        const int2 job = __ldg(m.fjob + i);
-        const int end = job.x + hi16(job.y), dst = lo16(job.y);
-        double acc = 0.0, acc2 = 0.0;
-        int q = job.x;
-        for (; q + 1 < end; q += 2) {
-            acc += gather_entry(m, q, c.rs);
-            acc2 += gather_entry(m, q + 1, c.rs);
-        }
-        if (q < end) acc += gather_entry(m, q, c.rs);
-        if (G == 32 || dst < m.n) fs[dst] = acc + acc2;  // one-warp cells have no split sums
-        else fp[dst - m.n] = acc + acc2;
-    }
+    const bool two = c.halves(m);
+    if (two) gather_terms<G, true>(m, c.rs, fs, fp, c.fb, lane);
+    else gather_terms<G, false>(m, c.rs, fs, fp, nullptr, lane);
     gsync<G>(gm);
     if (G > 32 && m.n_fsplit > 0) {  // split sums: their partials in a fixed order
         for (int i = lane; i < m.n_fsplit; i += G) {
             const int2 sp = __ldg(m.fsplit + i);
             const int first = lo16(sp.y), cnt = hi16(sp.y);
             double t = 0.0;
-            for (int j = 0; j < cnt; j++) t += fp[first + j];
+#pragma unroll 1
+            for (int j = 0; j < cnt; j++) t += two ? fp[first + j] + c.fb[m.n + first + j] : fp[first + j];
             fs[sp.x] = t;
+            if (two) c.fb[sp.x] = 0.0;
         }
         gsync<G>(gm);
     }
+}
+template <int G, int NPL, typename LT>
+__device__ __forceinline__ void take_f(const DevMech &m, const CellPtr<LT> &c, double (&f)[NPL], int lane) {
 #pragma unroll
     for (int s = 0; s < NPL; s++) {
-        int p = lane + G * s;
-        f[s] = (p < m.n) ? fs[p] : 0.0;
+        const int p = lane + G * s;
+        f[s] = p < m.n ? c.ys[p] : 0.0;
     }
-    gsync<G>(gm);
-}
-
-// y (own positions, registers) -> f (own positions)
-template <int G, int NPL, typename LT, bool W>
-__device__ __forceinline__ void eval_f(const DevMech &m, const CellPtr<LT> &c, const double (&y)[NPL],
-                                       double (&f)[NPL], int lane, unsigned gm) {
+    if (c.halves(m)) {
 #pragma unroll
-    for (int s = 0; s < NPL; s++) {
-        int p = lane + G * s;
-        if (p < m.n) c.ys[p] = y[s];
+        for (int s = 0; s < NPL; s++) {
+            const int p = lane + G * s;
+            if (p < m.n) f[s] += c.fb[p];
+        }
     }
-    gsync<G>(gm);
-    eval_f_ys<G, NPL, LT, W>(m, c, f, lane, gm);
+}
+// the same, out of line: the evaluations outside the Newton loop (a call's
+// first two, a restart's) share one copy of the code, so that the loop's own
+// stays in the instruction cache
+template <int G, typename LT, bool W>
+__device__ __noinline__ void eval_f_call(const DevMech &m, int base, int lane, unsigned gm) {
+    const CellPtr<LT> c(base, m);
+    eval_f_ys<G, LT, W>(m, c, lane, gm);
 }
 
-// f at y = a + b u (own positions), without a register copy of y
+// f at y = a + b u (own positions), out of line
 template <int G, int NPL, typename LT, bool W>
 __device__ __forceinline__ void eval_f_at(const DevMech &m, const CellPtr<LT> &c, const double (&a)[NPL],
                                           double b, const double (&u)[NPL], double (&f)[NPL], int lane,
@@ -552,7 +655,39 @@ __device__ __forceinline__ void eval_f_at(const DevMech &m, const CellPtr<LT> &c
         if (p < m.n) c.ys[p] = a[s] + b * u[s];
     }
     gsync<G>(gm);
-    eval_f_ys<G, NPL, LT, W>(m, c, f, lane, gm);
+    eval_f_call<G, LT, W>(m, c.base, lane, gm);
+    take_f<G, NPL, LT>(m, c, f, lane);
+}
+
+// f at y (own positions), out of line
+template <int G, int NPL, typename LT, bool W>
+__device__ __forceinline__ void eval_f(const DevMech &m, const CellPtr<LT> &c, const double (&y)[NPL],
+                                       double (&f)[NPL], int lane, unsigned gm) {
+#pragma unroll
+    for (int s = 0; s < NPL; s++) {
+        int p = lane + G * s;
+        if (p < m.n) c.ys[p] = y[s];
+    }
+    gsync<G>(gm);
+    eval_f_call<G, LT, W>(m, c.base, lane, gm);
+    take_f<G, NPL, LT>(m, c, f, lane);
+}
+
+// f at y = z + e (own positions), e zero in a step's first iteration
+template <int G, int NPL, typename LT, bool W>
+__device__ __forceinline__ void eval_f_newton(const DevMech &m, const CellPtr<LT> &c, const double (&z)[NPL],
+                                              const double (&e)[NPL], bool first, double (&f)[NPL], int lane,
+                                              unsigned gm) {
+#pragma unroll
+    for (int s = 0; s < NPL; s++) {
+        int p = lane + G * s;
+        double y = z[s];
+        if (!first) y += e[s];
+        if (p < m.n) c.ys[p] = y;
+    }
+    gsync<G>(gm);
+    eval_f_ys<G, LT, W>(m, c, lane, gm);
+    take_f<G, NPL, LT>(m, c, f, lane);
 }
 
 // ---- Jacobian gather: J (or M = I - gamma J) at ys into LU storage -----------
@@ -584,17 +719,20 @@ __device__ __forceinline__ void assemble(const DevMech &m, const CellPtr<LT> &c,
         if constexpr (W) {
             water_constants(kf32, kr32);
         } else {
-            for (int k = lane; k < m.R; k += G) kf32[k] = (LT)c.kf[k];
-            for (int k = lane; k < m.n_rev; k += G) kr32[k] = (LT)c.kr[k];
+#pragma unroll 1
+            for (int k = lane; k < m.R; k += G) kf32[k] = to_lu<LT>(c.kf[k]);
+#pragma unroll 1
+            for (int k = lane; k < m.n_rev; k += G) kr32[k] = to_lu<LT>(c.kr[k]);
         }
         // y to FP32 in place, G positions at a time: a chunk's FP32 values
         // overwrite only FP64 values of this or earlier chunks, and the
         // group reads its chunk before any lane writes it
+#pragma unroll 1
         for (int b0 = 0; b0 < m.n; b0 += G) {
             const int p = b0 + lane;
             const double v = p < m.n ? c.ys[p] : 0.0;
             gsync<G>(gm);
-            if (p < m.n) y32[p] = (LT)v;
+            if (p < m.n) y32[p] = to_lu<LT>(v);
         }
         kfv = kf32;
         krv = kr32;
@@ -616,52 +754,45 @@ __device__ __forceinline__ void assemble(const DevMech &m, const CellPtr<LT> &c,
         float4 *z4 = (float4 *)c.lu;
         const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
         const int nv = m.nlu / V;
+#pragma unroll 1
         for (int i = lane; i < nv; i += G) z4[i] = zero;
         for (int i = nv * V + lane; i < m.nlu; i += G) c.lu[i] = (LT)0;
     }
     gsync<G>(gm);
+    // flat per-lane entry lists: coalesced records read one step ahead, one
+    // store per non-zero
     const LT g = (LT)gamma;
-    if constexpr (sizeof(LT) == 4) {
-        {
-            // flat per-lane entry list: independent loads, one store per non-zero
-            const int b = __ldg(m.jl_ptr + lane), e = __ldg(m.jl_ptr + lane + 1);
-            LT acc = (LT)0;
-#pragma unroll 4
-            for (int i = b; i < e; i++) {
-                const int4 r = __ldg(m.jl_rec + i);
-                const int k = (int)(short)(r.y & 0xffff);
-                const int o1 = hi16(r.y), o2 = lo16(r.w);
-                LT v = __int_as_float(r.x) * (k >= 0 ? kfv[k] : krv[-k - 1]);
-                if (o1 != NONE16) v *= yv[o1];
-                if (o2 != NONE16) v *= yv[o2];
-                acc += v;
-                if (r.z & (1 << 17)) {
-                    if (mode == 0)
-                        c.lu[r.z & 0xffff] = ((r.z >> 16) & 1 ? (LT)1 : (LT)0) - g * acc;
-                    else
-                        out[hi16(r.w)] = (double)acc;
-                    acc = (LT)0;
-                }
-            }
+    const int4 *rec = m.jls + lane;
+    const double *cf = m.jlc + lane;
+    LT acc = (LT)0;
+    int4 r = __ldg(rec);
+    const int steps = m.n_jstep[G > 32 ? lane >> 5 : 0];
+#pragma unroll 1
+    for (int i = 0; i < steps; i++) {
+        rec += G;
+        int4 rn = make_int4(0, (int)0xffff0000u, 1 << 18, 0xffff);  // a lane past its list reads no more
+        if (!(r.z & (1 << 18))) rn = __ldg(rec);
+        const int k = (int)(short)(r.y & 0xffff);
+        const int o1 = hi16(r.y), o2 = lo16(r.w);
+        LT v;
+        if constexpr (sizeof(LT) == 4) v = __int_as_float(r.x);
+        else v = r.z & (1 << 18) && !(r.z & (1 << 17)) ? (LT)0 : (LT)__ldg(cf);
+        cf += G;
+        const LT *kp = k >= 0 ? kfv + k : krv + (-k - 1);
+        const LT kv = *kp, y1 = yv[o1 != NONE16 ? o1 : 0], y2 = yv[o2 != NONE16 ? o2 : 0];
+        v *= kv;
+        if (o1 != NONE16) v *= y1;
+        if (o2 != NONE16) v *= y2;
+        acc += v;
+        const bool end = r.z & (1 << 17);
+        if (mode == 0) {
+            const LT M = ((r.z >> 16) & 1 ? (LT)1 : (LT)0) - g * acc;
+            if (end) c.lu[r.z & 0xffff] = M;
+        } else {
+            if (end) out[hi16(r.w)] = (double)acc;
         }
-    }
-    if constexpr (sizeof(LT) == 8) {  // FP64: one non-zero per lane at a time
-        for (int t = lane; t < m.nnzJ; t += G) {
-            LT acc = (LT)0;
-            const int4 nz = __ldg(m.jnz + t);
-            for (int q = nz.x; q < nz.y; q++) {
-                const int k = __ldg(m.jk + q);
-                LT v = (LT)__ldg(m.jc + q) * (k >= 0 ? kfv[k] : krv[-k - 1]);
-                const int o1 = __ldg(m.jo + 2 * q), o2 = __ldg(m.jo + 2 * q + 1);
-                if (o1 >= 0) v *= yv[o1];
-                if (o2 >= 0) v *= yv[o2];
-                acc += v;
-            }
-            if (mode == 0)
-                c.lu[nz.z] = (nz.w ? (LT)1 : (LT)0) - g * acc;
-            else
-                out[t] = (double)acc;
-        }
+        acc = end ? (LT)0 : acc;
+        r = rn;
     }
     gsync<G>(gm);
     if constexpr (W) {
@@ -686,136 +817,177 @@ __device__ __forceinline__ bool bad_pivot(LT u) {
     return !(fabs(u) > tiny_pivot<LT>()) || !isfinite(u);
 }
 
-// Dense trailing block, right-looking in panels of W pivots.  For each
-// panel: (1) factor its W columns over the rows below (lane l owns rows
-// l + 32 t); (2) forward-substitute the W pivot rows to the right of the
-// panel with the panel's unit lower triangle (lane l owns columns l + 32 t);
-// (3) one rank-W update of the trailing block, each entry loaded and stored
-// once per panel (the W multipliers of a row are broadcast loads).
+// f(integral_constant NS) for a dense block of D rows, NS = rows per lane of
+// its warp (at most 4; a cell of at most MAXN positions has no more)
+template <int V> struct IntC { static constexpr int value = V; };
+template <int MAXN, class F>
+__device__ __forceinline__ void dense_rows(int D, F f) {
+    constexpr int TOP = MAXN >= 128 ? 4 : (MAXN + 31) / 32;
+    const int ns = (D + 31) >> 5;
+    if (ns == 0) return;
+    if (TOP == 1 || ns == 1) f(IntC<1>());
+    else if (TOP == 2 || ns == 2) f(IntC<(TOP >= 2 ? 2 : 1)>());
+    else if (TOP == 3 || ns == 3) f(IntC<(TOP >= 3 ? 3 : 1)>());
+    else f(IntC<(TOP >= 4 ? 4 : 1)>());
+}
+
+// 16-byte pieces of the dense block's rows (4 FP32 or 2 FP64 values)
+template <typename LT> struct Vec16;
+template <> struct Vec16<float> {
+    static constexpr int N = 4;
+    static __device__ __forceinline__ void ld(const float *p, float (&v)[4]) {
+        const float4 t = *reinterpret_cast<const float4 *>(p);
+        v[0] = t.x; v[1] = t.y; v[2] = t.z; v[3] = t.w;
+    }
+    static __device__ __forceinline__ void st(float *p, const float (&v)[4]) {
+        *reinterpret_cast<float4 *>(p) = make_float4(v[0], v[1], v[2], v[3]);
+    }
+};
+template <> struct Vec16<double> {
+    static constexpr int N = 2;
+    static __device__ __forceinline__ void ld(const double *p, double (&v)[2]) {
+        const double2 t = *reinterpret_cast<const double2 *>(p);
+        v[0] = t.x; v[1] = t.y;
+    }
+    static __device__ __forceinline__ void st(double *p, const double (&v)[2]) {
+        *reinterpret_cast<double2 *>(p) = make_double2(v[0], v[1]);
+    }
+};
+
+// Dense trailing block, right-looking in panels of DENSE_W pivots, lane l
+// owning rows l + 32 t.  For each panel: (1) its columns are factored in the
+// owners' registers, the pivot row's entries broadcast by shuffles, so that a
+// pivot's chain is a shuffle, a reciprocal and two operations; (2) the pivot
+// rows right of the panel are forward-substituted with the panel's unit lower
+// triangle (lane l takes columns l + 32 s); (3) one rank-DENSE_W update of
+// the trailing rows, 16 bytes of a row at a time, the multipliers already in
+// registers and the pivot rows broadcast.  The row stride is 4 mod 8 values,
+// so that 16-byte accesses of FP32 rows spread over all banks.  Every entry
+// takes its updates one by one in pivot order, as a plain elimination does.
 // Pivots are checked and replaced by their reciprocals.
-template <int NS, int W, typename LT>
-__device__ __forceinline__ bool dense_factor(LT *A, int D, int LD, int lane, unsigned gm) {
+constexpr int DENSE_W = 8;
+template <int NS, typename LT>
+__device__ __noinline__ bool dense_factor(LT *A, int D, int LD, int lane, unsigned gm) {
+    using V = Vec16<LT>;
+    constexpr int N = V::N, W = DENSE_W;
     bool bad = false;
-    for (int kp = 0; kp < D; kp += W) {
-        const int w = min(W, D - kp);
-        // (1) panel columns kp .. kp+w-1
-        for (int c = 0; c < w; c++) {
-            const int k = kp + c;
-            const LT piv = A[k * LD + k];
-            bad |= bad_pivot(piv);
-            const LT rp = recip(piv);
-            LT uk[W];  // the pivot row inside the panel
 #pragma unroll
-            for (int j = 1; j < W; j++) uk[j] = (c + j < w) ? A[k * LD + k + j] : (LT)0;
+    for (int kb = 0; kb < NS; kb++) {
+        const int k1 = min(D, 32 * kb + 32);
+#pragma unroll 1
+        for (int kp = 32 * kb; kp < k1; kp += W) {
+            const int o = kp - 32 * kb;  // the panel's first row among the owners
+            // (1) panel columns kp .. kp+W-1 of the rows from 32 kb on
+            LT a[NS][W];
 #pragma unroll
-            for (int t = 0; t < NS; t++) {
-                const int i = lane + 32 * t;
-                if (i > k && i < D) {
-                    LT *row = A + i * LD;
-                    const LT l = row[k] * rp;
-                    row[k] = l;
+            for (int t = kb; t < NS; t++) {
+                const LT *row = A + min(lane + 32 * t, D - 1) * LD + kp;
 #pragma unroll
-                    for (int j = 1; j < W; j++)
-                        if (c + j < w) row[k + j] -= l * uk[j];
+                for (int v = 0; v < W; v += N) {
+                    LT x[N] = {};
+                    if (kp + v < LD) V::ld(row + v, x);
+#pragma unroll
+                    for (int i = 0; i < N; i++) a[t][v + i] = x[i];
+                }
+            }
+#pragma unroll
+            for (int c = 0; c < W; c++) {
+                if (kp + c < D) {
+                    LT p[W];
+#pragma unroll
+                    for (int j = c; j < W; j++) p[j] = __shfl_sync(gm, a[kb][j], o + c);
+                    bad |= bad_pivot(p[c]);
+                    const LT rp = recip(p[c]);
+#pragma unroll
+                    for (int t = kb; t < NS; t++) {
+                        if (t > kb || lane > o + c) {
+                            const LT l = a[t][c] * rp;
+                            a[t][c] = l;
+#pragma unroll
+                            for (int j = c + 1; j < W; j++) a[t][j] -= l * p[j];
+                        }
+                    }
+                    if (lane == o + c) a[kb][c] = rp;
+                }
+            }
+#pragma unroll
+            for (int t = kb; t < NS; t++) {
+                if ((t > kb || lane >= o) && lane + 32 * t < D) {
+                    LT *row = A + (lane + 32 * t) * LD + kp;
+#pragma unroll
+                    for (int v = 0; v < W; v += N) {
+                        LT x[N];
+#pragma unroll
+                        for (int i = 0; i < N; i++) x[i] = a[t][v + i];
+                        if (kp + v < LD) V::st(row + v, x);
+                    }
                 }
             }
             __syncwarp(gm);
-            if (lane == 0) A[k * LD + k] = rp;
-        }
-        const int j0 = kp + w;
-        if (j0 >= D) break;
-        // (2) pivot rows of the panel, columns right of it: unit lower solve
-        LT u[W][NS];
-        bool act[NS];
+            const int j0 = kp + W;
+            if (j0 >= D) break;
+            // (2) pivot rows of the panel, columns right of it
+            LT tr[W][W];
 #pragma unroll
-        for (int t = 0; t < NS; t++) {
-            const int j = j0 + lane + 32 * t;
-            act[t] = j < D;
+            for (int r = 1; r < W; r++) {
 #pragma unroll
-            for (int r = 0; r < W; r++) {
-                LT v = (LT)0;
-                if (act[t] && r < w) {
-                    v = A[(kp + r) * LD + j];
+                for (int v = 0; v < r; v += N) {
+                    LT x[N];
+                    V::ld(A + (kp + r) * LD + kp + v, x);
 #pragma unroll
-                    for (int p = 0; p < r; p++) v -= A[(kp + r) * LD + kp + p] * u[p][t];
-                    A[(kp + r) * LD + j] = v;
-                }
-                u[r][t] = v;
-            }
-        }
-        __syncwarp(gm);
-        // (3) trailing block: rank-w update, two rows at a time with every
-        // load issued before the stores (rows never alias; the compiler
-        // cannot know that)
-        int i = j0;
-        for (; i + 1 < D; i += 2) {
-            const LT *l0p = A + i * LD + kp, *l1p = l0p + LD;
-            LT l0[W], l1[W], a0[NS], a1[NS];
-#pragma unroll
-            for (int r = 0; r < W; r++) {
-                l0[r] = r < w ? l0p[r] : (LT)0;
-                l1[r] = r < w ? l1p[r] : (LT)0;
-            }
-#pragma unroll
-            for (int t = 0; t < NS; t++) {
-                const int col = j0 + lane + 32 * t;
-                a0[t] = act[t] ? A[i * LD + col] : (LT)0;
-                a1[t] = act[t] ? A[(i + 1) * LD + col] : (LT)0;
-            }
-#pragma unroll
-            for (int t = 0; t < NS; t++) {
-#pragma unroll
-                for (int r = 0; r < W; r++) {
-                    a0[t] -= l0[r] * u[r][t];
-                    a1[t] -= l1[r] * u[r][t];
+                    for (int i = 0; i < N; i++) tr[r][v + i] = x[i];
                 }
             }
+#pragma unroll 1
+            for (int j = j0 + lane; j < D; j += 32) {
+                LT u[W];
 #pragma unroll
-            for (int t = 0; t < NS; t++) {
-                if (act[t]) {
-                    const int col = j0 + lane + 32 * t;
-                    A[i * LD + col] = a0[t];
-                    A[(i + 1) * LD + col] = a1[t];
+                for (int r = 0; r < W; r++) u[r] = A[(kp + r) * LD + j];
+#pragma unroll
+                for (int r = 1; r < W; r++) {
+#pragma unroll
+                    for (int p = 0; p < r; p++) u[r] -= tr[r][p] * u[p];
+                }
+#pragma unroll
+                for (int r = 1; r < W; r++) A[(kp + r) * LD + j] = u[r];
+            }
+            __syncwarp(gm);
+            // (3) trailing rows
+#pragma unroll 1
+            for (int j = j0; j < D; j += N) {
+                LT u[W][N];
+#pragma unroll
+                for (int r = 0; r < W; r++) V::ld(A + (kp + r) * LD + j, u[r]);
+#pragma unroll
+                for (int t = kb; t < NS; t++) {
+                    if (t > kb || o + W < 32) {
+                        LT *row = A + min(lane + 32 * t, D - 1) * LD + j;
+                        LT x[N];
+                        V::ld(row, x);
+#pragma unroll
+                        for (int r = 0; r < W; r++) {
+#pragma unroll
+                            for (int i = 0; i < N; i++) x[i] -= a[t][r] * u[r][i];
+                        }
+                        if ((t > kb || lane >= o + W) && lane + 32 * t < D) V::st(row, x);
+                    }
                 }
             }
         }
-        if (i < D) {  // odd number of trailing rows: the last one alone
-            const LT *l0p = A + i * LD + kp;
-            LT l0[W];
-#pragma unroll
-            for (int r = 0; r < W; r++) l0[r] = r < w ? l0p[r] : (LT)0;
-#pragma unroll
-            for (int t = 0; t < NS; t++) {
-                if (act[t]) {
-                    LT *a = A + i * LD + j0 + lane + 32 * t;
-                    LT v = *a;
-#pragma unroll
-                    for (int r = 0; r < W; r++) v -= l0[r] * u[r][t];
-                    *a = v;
-                }
-            }
-        }
-        __syncwarp(gm);
     }
     return bad;
 }
 
-// panel width of the dense factorisation
-constexpr int DENSE_W = 8;
-
 // one op of the row-wise factorisation: a division makes the multiplier l
-// (lu[src] holds 1 / U(k,k)), an update subtracts l U(k,j) from its target,
-// an LU value or (bit 15 of the target; block cells only) a partial sum
-template <bool PART, typename LT>
-__device__ __forceinline__ void factor_op(uint32_t op, LT *lu, LT *part, int pbase, LT &l) {
+// (lu[src] holds 1 / U(k,k)), an update subtracts l U(k,j) from its target
+template <typename LT>
+__device__ __forceinline__ void factor_op(uint32_t op, LT *lu, LT &l) {
     const int t = CAMP_OP_TGT(op), s = CAMP_OP_SRC(op);
     if (op & CAMP_OP_DIV) {
         l = lu[t] * lu[s];
         lu[t] = l;
-    } else if (PART && (t & 0x8000)) {
-        part[pbase + (t & 0x7fff)] -= l * lu[s];
     } else {
-        lu[t] -= l * lu[s];
+        lu[t] = fma(-l, lu[s], lu[t]);
     }
 }
 
@@ -827,23 +999,42 @@ __device__ __forceinline__ bool take_reciprocal(const DevMech &m, LT *lu, int i)
     return bad_pivot(u);
 }
 
-template <int G, typename LT>
+template <int G, int NPL, typename LT>
 __device__ bool factor(const DevMech &m, const CellPtr<LT> &c, int lane, unsigned gm) {
     LT *lu = c.lu;
     LT *part = (LT *)(c.rs + m.R);  // chunk partials: the rate scratch is free here
     bool bad = false;
-    // sparse rows (and the sparse-pivot updates of the block rows), by level
+    // sparse rows (and the sparse-pivot updates of the block rows), by level:
+    // each lane runs through its op list, the next op's word read ahead
+#pragma unroll 1
     for (int L = 0; L < m.n_flev; L++) {
-        const int b = __ldg(m.ljob_ptr + L), e = __ldg(m.ljob_ptr + L + 1);
-        for (int r = b + lane; r < e; r += G) {
-            const int4 jb = __ldg(m.ljob + r);
-            const int cnt = lo16(jb.y);
-            if constexpr (G > 32) {
-                for (int k = 0; k < hi16(jb.y); k++) part[jb.w + k] = (LT)0;
+        const int b = __ldg(m.fst_ptr + L), e = __ldg(m.fst_ptr + L + 1);
+        if constexpr (G > 32) {
+            const int np = __ldg(m.fst_part + L);
+            if (np > 0) {
+                for (int k = lane; k < np; k += G) part[k] = (LT)0;
+                gsync<G>(gm);
             }
-            LT l = (LT)0;
-            for (int q = jb.x; q < jb.x + cnt; q++) factor_op<(G > 32)>(__ldg(m.lops + q), lu, part, jb.w, l);
-            if (hi16(jb.z) & 1) bad |= take_reciprocal(m, lu, lo16(jb.z));
+        }
+        const uint32_t *ops = m.fst + (size_t)b * G + lane;
+        LT l = (LT)0;
+        uint32_t op = __ldg(ops);
+#pragma unroll 1
+        for (int q = b; q < e; q++) {
+            ops += G;
+            const uint32_t next = __ldg(ops);  // one step of padding follows the last
+            const int t = CAMP_OP_TGT(op), s = CAMP_OP_SRC(op);
+            const bool div = (op & CAMP_OP_DIV) != 0, act = s != CAMP_OP_NOSRC, pivot = !act && !div;
+            LT *to = (G > 32 && (t & 0x8000) && !div) ? part + (t & 0x7fff) : lu + t;
+            const LT tv = *to, sv = lu[act ? s : 0];
+            const LT upd = fma(-l, sv, tv), quot = tv * sv;
+            l = div ? quot : l;
+            if (act) *to = div ? quot : upd;
+            if (pivot) {  // the row's pivot
+                *to = recip(tv);
+                bad |= bad_pivot(tv);
+            }
+            op = next;
         }
         gsync<G>(gm);
         if constexpr (G > 32) {  // rows cut into chunks: partials in order, then the tail
@@ -859,7 +1050,7 @@ __device__ bool factor(const DevMech &m, const CellPtr<LT> &c, int lane, unsigne
                 }
                 const int2 tl = __ldg(m.ltail + k);
                 LT l = (LT)0;
-                for (int q = tl.x; q < tl.x + tl.y; q++) factor_op<false>(__ldg(m.lops + q), lu, part, 0, l);
+                for (int q = tl.x; q < tl.x + tl.y; q++) factor_op(__ldg(m.lops + q), lu, l);
                 if (hi16(rd.x) & 1) bad |= take_reciprocal(m, lu, lo16(rd.x));
             }
             if (re > rb) gsync<G>(gm);
@@ -869,193 +1060,190 @@ __device__ bool factor(const DevMech &m, const CellPtr<LT> &c, int lane, unsigne
     LT *A = lu + m.dbase;
     if (G <= 32 || lane < 32) {
         const unsigned wm = G <= 32 ? gm : 0xffffffffu;
-        switch ((m.D + 31) >> 5) {
-        case 0: break;
-        case 1: bad |= dense_factor<1, DENSE_W, LT>(A, m.D, m.LD, lane, wm); break;
-        case 2: bad |= dense_factor<2, DENSE_W, LT>(A, m.D, m.LD, lane, wm); break;
-        case 3: bad |= dense_factor<3, DENSE_W, LT>(A, m.D, m.LD, lane, wm); break;
-        default: bad |= dense_factor<4, DENSE_W, LT>(A, m.D, m.LD, lane, wm); break;
-        }
+        dense_rows<G * NPL>(m.D, [&](auto ns) { bad |= dense_factor<decltype(ns)::value, LT>(A, m.D, m.LD, lane, wm); });
     }
     return !gany<G>(bad, gm);
 }
 
 // ---- substitution: solves (LU) x = x in place (c.x holds the right side) -----
 // Sparse rows go level by level through shared memory.  The dense block's
-// right side lives in registers (lane l holds rows l + 32 t); each pivot's
-// value is broadcast with a shuffle, and the loops run one 32-row diagonal
-// block at a time so that only that block's rows need a comparison.  Rows
-// past the block end read the last row (a valid address) and are discarded.
-template <int NS, typename LT, int SP>
-__device__ __forceinline__ void dense_subst(const LT *A, int D, int LD, LT *xb, int lane, unsigned gm) {
-    LT xr[NS];
-    int rowc[NS];
+// right side lives in registers (lane l holds rows l + 32 t), and the loops
+// run one 32-row diagonal block at a time so that only that block's rows
+// need a comparison.  Rows past the block end read the last row (a valid
+// address) and are discarded.
+//
+// FP32: four pivots a round.  Their not yet final values come by independent
+// shuffles, every lane finishes them with the broadcast 4 x 4 diagonal block,
+// then the four columns, 16 bytes of a row at a time, update the rows: a
+// round's chain is one shuffle and about a dozen FP32 operations.  The rows of
+// the diagonal block take the same operations in the same order in their
+// owner lanes as in the broadcast triangle; the backward pass scales them by
+// their reciprocal pivots at the end.  (Eight pivots a round have a shorter
+// chain per pivot but half again as many instructions: slower at full
+// occupancy.)
+template <int NS, int KB>
+__device__ __forceinline__ void forward_block(const float *A, int D, int LD, const float *const (&row)[NS],
+                                              float (&xr)[NS], int lane, unsigned gm) {
+    using V = Vec16<float>;
+    const int k0 = 32 * KB, k1 = min(D, k0 + 32);
+    const float *dg = A + k0 * (LD + 1);
+    int k = k0;
+#pragma unroll 1
+    for (; k + 4 <= k1; k += 4, dg += 4 * (LD + 1)) {
+        const int o = k - k0, in = lane - o;
+        float a[NS][4], d1[4], d2[4], d3[4], x[4];
+        V::ld(dg + LD, d1);
+        V::ld(dg + 2 * LD, d2);
+        V::ld(dg + 3 * LD, d3);
+#pragma unroll
+        for (int t = KB; t < NS; t++) V::ld(row[t] + k, a[t]);
+#pragma unroll
+        for (int p = 0; p < 4; p++) x[p] = __shfl_sync(gm, xr[KB], o + p);
+        x[1] -= d1[0] * x[0];
+        x[2] -= d2[0] * x[0];
+        x[2] -= d2[1] * x[1];
+        x[3] -= d3[0] * x[0];
+        x[3] -= d3[1] * x[1];
+        x[3] -= d3[2] * x[2];
+#pragma unroll
+        for (int p = 0; p < 4; p++) {
+            if (in > p) xr[KB] -= a[KB][p] * x[p];
+#pragma unroll
+            for (int t = KB + 1; t < NS; t++) xr[t] -= a[t][p] * x[p];
+        }
+    }
+#pragma unroll 1
+    for (; k < k1; k++) {  // the block's last pivots, one at a time
+        const int o = k - k0;
+        const float xk = __shfl_sync(gm, xr[KB], o);
+#pragma unroll
+        for (int t = KB; t < NS; t++) {
+            const float a = row[t][k];
+            if (t > KB || lane > o) xr[t] -= a * xk;
+        }
+    }
+    if constexpr (KB + 1 < NS) forward_block<NS, KB + 1>(A, D, LD, row, xr, lane, gm);
+}
+template <int NS, int KB>
+__device__ __forceinline__ void backward_block(const float *A, int D, int LD, const float *const (&row)[NS],
+                                               float (&xr)[NS], int lane, unsigned gm) {
+    using V = Vec16<float>;
+    const int k0 = 32 * KB, k1 = min(D, k0 + 32);
+    int k = k1;  // one past the next pivot
+#pragma unroll 1
+    for (; k > k0 && (k & 3); k--) {  // the ragged end, one pivot at a time
+        const int o = k - 1 - k0;
+        const float xk = __shfl_sync(gm, xr[KB], o) * A[(k - 1) * LD + k - 1];
+#pragma unroll
+        for (int t = 0; t <= KB; t++) {
+            const float a = row[t][k - 1];
+            if (t < KB || lane < o) xr[t] -= a * xk;
+        }
+    }
+    k -= 4;
+    const float *dg = A + k * (LD + 1);
+#pragma unroll 1
+    for (; k >= k0; k -= 4, dg -= 4 * (LD + 1)) {  // k0 is a multiple of 4
+        const int o = k - k0, in = lane - o;
+        float a[NS][4], d[4][4], x[4];
+#pragma unroll
+        for (int p = 0; p < 4; p++) V::ld(dg + p * LD, d[p]);
+#pragma unroll
+        for (int t = 0; t <= KB; t++) V::ld(row[t] + k, a[t]);
+#pragma unroll
+        for (int p = 0; p < 4; p++) x[p] = __shfl_sync(gm, xr[KB], o + p);
+#pragma unroll
+        for (int p = 3; p >= 0; p--) {
+#pragma unroll
+            for (int q = 3; q > p; q--) x[p] -= d[p][q] * x[q];
+            x[p] *= d[p][p];
+        }
+#pragma unroll
+        for (int p = 3; p >= 0; p--) {
+            if (in < p) xr[KB] -= a[KB][p] * x[p];
+#pragma unroll
+            for (int t = 0; t < KB; t++) xr[t] -= a[t][p] * x[p];
+        }
+    }
+    xr[KB] *= row[KB][min(lane + k0, D - 1)];  // final up to the reciprocal pivots
+    if constexpr (KB > 0) backward_block<NS, KB - 1>(A, D, LD, row, xr, lane, gm);
+}
+template <int NS>
+__device__ __forceinline__ void dense_subst(const float *A, int D, int LD, float *xb, int lane, unsigned gm) {
+    float xr[NS];
+    const float *row[NS];
 #pragma unroll
     for (int t = 0; t < NS; t++) {
         const int i = lane + 32 * t;
-        rowc[t] = (i < D ? i : D - 1) * LD;
-        xr[t] = i < D ? xb[i] : (LT)0;
+        row[t] = A + min(i, D - 1) * LD;
+        xr[t] = i < D ? xb[i] : 0.0f;
     }
-    if constexpr (SP == 2) {
-    // forward, unit lower, two pivots per round: x_k and the not yet final
-    // x_{k+1} come by two independent shuffles, every lane finishes x_{k+1}
-    // with the broadcast L(k+1,k), then both columns update the rows below
+    forward_block<NS, 0>(A, D, LD, row, xr, lane, gm);
+    backward_block<NS, NS - 1>(A, D, LD, row, xr, lane, gm);
 #pragma unroll
-    for (int kb = 0; kb < NS; kb++) {
-        const int k0 = 32 * kb, k1 = min(D, k0 + 32);
-        int k = k0;
-#pragma unroll 2
-        for (; k + 1 < k1; k += 2) {
-            const int o = k - k0;
-            const LT xk = __shfl_sync(gm, xr[kb], o);
-            const LT xn = __shfl_sync(gm, xr[kb], o + 1);
-            const LT l10 = A[(k + 1) * LD + k];
-            const LT xk1 = xn - l10 * xk;
-#pragma unroll
-            for (int t = kb; t < NS; t++) {
-                const LT a0 = A[rowc[t] + k], a1 = A[rowc[t] + k + 1];
-                if (t > kb || lane > o + 1) {
-                    xr[t] -= a0 * xk;
-                    xr[t] -= a1 * xk1;
-                } else if (lane == o + 1) {
-                    xr[t] = xk1;
-                }
-            }
-        }
-        if (k < k1) {  // odd block length: one pivot left
-            const int o = k - k0;
-            const LT xk = __shfl_sync(gm, xr[kb], o);
-#pragma unroll
-            for (int t = kb; t < NS; t++) {
-                const LT a = A[rowc[t] + k];
-                if (t > kb || lane > o) xr[t] -= a * xk;
-            }
-        }
+    for (int t = 0; t < NS; t++) {
+        const int i = lane + 32 * t;
+        if (i < D) xb[i] = xr[t];
     }
-    // backward, upper with reciprocal diagonal, two pivots per round
+}
+
+// FP64: bound by the FP64 port, so one pivot at a time without redundant
+// products; two columns of a row per load.
+template <int NS>
+__device__ __forceinline__ void dense_subst(const double *A, int D, int LD, double *xb, int lane, unsigned gm) {
+    using V = Vec16<double>;
+    double xr[NS];
+    const double *row[NS];
 #pragma unroll
-    for (int kb = NS - 1; kb >= 0; kb--) {
-        const int k0 = 32 * kb, k1 = min(D, k0 + 32);
-        int k = k1 - 1;
-#pragma unroll 2
-        for (; k - 1 >= k0; k -= 2) {
-            const int o = k - k0;  // pivots k and k-1
-            const LT xk = __shfl_sync(gm, xr[kb], o) * A[k * LD + k];
-            const LT xp = __shfl_sync(gm, xr[kb], o - 1);
-            const LT xk1 = (xp - A[(k - 1) * LD + k] * xk) * A[(k - 1) * LD + k - 1];
-#pragma unroll
-            for (int t = 0; t <= kb; t++) {
-                const LT a0 = A[rowc[t] + k], a1 = A[rowc[t] + k - 1];
-                if (t < kb || lane < o - 1) {
-                    xr[t] -= a0 * xk;
-                    xr[t] -= a1 * xk1;
-                } else if (lane == o) {
-                    xr[t] = xk;
-                } else if (lane == o - 1) {
-                    xr[t] = xk1;
-                }
-            }
-        }
-        if (k >= k0) {  // one pivot left
-            const int o = k - k0;
-            const LT xk = __shfl_sync(gm, xr[kb], o) * A[k * LD + k];
-#pragma unroll
-            for (int t = 0; t <= kb; t++) {
-                const LT a = A[rowc[t] + k];
-                if (t < kb || lane < o) xr[t] -= a * xk;
-                else if (lane == o) xr[t] = xk;
-            }
-        }
+    for (int t = 0; t < NS; t++) {
+        const int i = lane + 32 * t;
+        row[t] = A + min(i, D - 1) * LD;
+        xr[t] = i < D ? xb[i] : 0.0;
     }
-    } else {
-    // forward, unit lower, SP pivots per round: the not yet final x_k ..
-    // x_{k+SP-1} come by independent shuffles, every lane finishes them with
-    // the broadcast L entries of the diagonal block (a chain SP-1 deep), then
-    // the SP columns update the rows below
 #pragma unroll
     for (int kb = 0; kb < NS; kb++) {
         const int k0 = 32 * kb, k1 = min(D, k0 + 32);
         int k = k0;
 #pragma unroll 1
-        for (; k + SP <= k1; k += SP) {
+        for (; k < k1; k += 2) {
             const int o = k - k0;
-            LT xf[SP];
+            double a[NS][2];
 #pragma unroll
-            for (int p = 0; p < SP; p++) xf[p] = __shfl_sync(gm, xr[kb], o + p);
+            for (int t = kb; t < NS; t++) V::ld(row[t] + k, a[t]);
+            const double x0 = __shfl_sync(gm, xr[kb], o);
 #pragma unroll
-            for (int p = 1; p < SP; p++) {
+            for (int t = kb; t < NS; t++)
+                if (t > kb || lane > o) xr[t] -= a[t][0] * x0;
+            if (k + 1 < k1) {
+                const double x1 = __shfl_sync(gm, xr[kb], o + 1);
 #pragma unroll
-                for (int q = 0; q < p; q++) xf[p] -= A[(k + p) * LD + k + q] * xf[q];
-            }
-#pragma unroll
-            for (int t = kb; t < NS; t++) {
-                LT a[SP];
-#pragma unroll
-                for (int p = 0; p < SP; p++) a[p] = A[rowc[t] + k + p];
-                if (t > kb || lane > o + SP - 1) {
-#pragma unroll
-                    for (int p = 0; p < SP; p++) xr[t] -= a[p] * xf[p];
-                } else {
-#pragma unroll
-                    for (int p = 1; p < SP; p++)
-                        if (lane == o + p) xr[t] = xf[p];
-                }
-            }
-        }
-        for (; k < k1; k++) {  // the block's last pivots, one at a time
-            const int o = k - k0;
-            const LT xk = __shfl_sync(gm, xr[kb], o);
-#pragma unroll
-            for (int t = kb; t < NS; t++) {
-                const LT a = A[rowc[t] + k];
-                if (t > kb || lane > o) xr[t] -= a * xk;
+                for (int t = kb; t < NS; t++)
+                    if (t > kb || lane > o + 1) xr[t] -= a[t][1] * x1;
             }
         }
     }
-    // backward, upper with reciprocal diagonal, SP pivots per round (k, k-1,
-    // ..., k-SP+1)
 #pragma unroll
     for (int kb = NS - 1; kb >= 0; kb--) {
         const int k0 = 32 * kb, k1 = min(D, k0 + 32);
-        int k = k1 - 1;
 #pragma unroll 1
-        for (; k - (SP - 1) >= k0; k -= SP) {
+        for (int k = (k1 - 1) & ~1; k >= k0; k -= 2) {  // columns k + 1 and k
             const int o = k - k0;
-            LT xf[SP];
+            double a[NS][2];
 #pragma unroll
-            for (int p = 0; p < SP; p++) xf[p] = __shfl_sync(gm, xr[kb], o - p);
+            for (int t = 0; t <= kb; t++) V::ld(row[t] + k, a[t]);
+            if (k + 1 < k1) {
+                const double x1 = __shfl_sync(gm, xr[kb], o + 1) * A[(k + 1) * LD + k + 1];
 #pragma unroll
-            for (int p = 0; p < SP; p++) {
-#pragma unroll
-                for (int q = 0; q < p; q++) xf[p] -= A[(k - p) * LD + k - q] * xf[q];
-                xf[p] *= A[(k - p) * LD + k - p];
+                for (int t = 0; t <= kb; t++)
+                    if (t < kb || lane < o + 1) xr[t] -= a[t][1] * x1;
             }
+            const double x0 = __shfl_sync(gm, xr[kb], o) * A[k * LD + k];
 #pragma unroll
-            for (int t = 0; t <= kb; t++) {
-                LT a[SP];
-#pragma unroll
-                for (int p = 0; p < SP; p++) a[p] = A[rowc[t] + k - p];
-                if (t < kb || lane < o - (SP - 1)) {
-#pragma unroll
-                    for (int p = 0; p < SP; p++) xr[t] -= a[p] * xf[p];
-                } else {
-#pragma unroll
-                    for (int p = 0; p < SP; p++)
-                        if (lane == o - p) xr[t] = xf[p];
-                }
-            }
+            for (int t = 0; t <= kb; t++)
+                if (t < kb || lane < o) xr[t] -= a[t][0] * x0;
         }
-        for (; k >= k0; k--) {  // one pivot at a time
-            const int o = k - k0;
-            const LT xk = __shfl_sync(gm, xr[kb], o) * A[k * LD + k];
-#pragma unroll
-            for (int t = 0; t <= kb; t++) {
-                const LT a = A[rowc[t] + k];
-                if (t < kb || lane < o) xr[t] -= a * xk;
-                else if (lane == o) xr[t] = xk;
-            }
-        }
-    }
+        const int i = lane + k0;
+        xr[kb] *= row[kb][min(i, D - 1)];
     }
 #pragma unroll
     for (int t = 0; t < NS; t++) {
@@ -1064,16 +1252,74 @@ __device__ __forceinline__ void dense_subst(const LT *A, int D, int LD, LT *xb, 
     }
 }
 
-// Pivots per round of the dense block's triangular solves for a cell shape
-// and LU precision: 4 for the FP32 LU of 8-slot lanes (measured:
-// multiphase-232 +3.6%, water parameter +2.0%; 8 cost it 1%), 2 otherwise
-// (4 cost the 3-slot gas-72 kernel 6.6% and the FP64 8-slot kernels 6-7%,
-// 3 cost gas-72 3.5%)
-template <int G, int NPL, typename LT>
-__host__ __device__ constexpr int subst_pivots() { return (sizeof(LT) == 4 && NPL >= 6) ? 4 : 2; }
+// The passes [p, pe) of a sparse substitution: in each, every lane takes one
+// row (DevMech::sub_pass), its entries two a step; the first entry of a pair
+// goes to the row's sum, the second to its odd accumulator.  The backward
+// pass scales the row by its reciprocal pivot.  The next pass's record, with
+// its first entries, and the next step's entries are read ahead, and operands
+// are loaded without branches (a missing entry reads entry 0), so that a
+// pass costs its chain of shared-memory loads alone.
+template <int G, typename LT, bool BACK>
+__device__ __forceinline__ void subst_passes(const DevMech &m, int p, int pe, const LT *lu, LT *x, LT *xp, int lane,
+                                             unsigned gm) {
+    if (p >= pe) return;
+    const int4 *rec = m.sub_pass + (size_t)p * G + lane;
+    int4 h = __ldg(rec);
+    int L = 0;
+#pragma unroll 1
+    for (; p < pe; p++) {
+        rec += G;
+        const int4 hn = __ldg(rec);  // one pass of padding follows the last
+        const int steps = h.w & 0xfff, i = lo16(h.x);
+        const int2 *ent = m.sub + (size_t)((unsigned)h.w >> 14) * G + lane;
+        int ea = h.y, eb = h.z;
+        LT *to = x + (h.x >= 0 ? i : 0);
+        LT s = *to, s2 = (LT)0;
+        if constexpr (!BACK && G > 32) {
+            if (h.x >= 0 && i >= m.n) {  // a chunk of a split row
+                to = xp + (i - m.n);
+                s = (LT)0;
+            }
+        }
+        LT dg = (LT)1;
+        if constexpr (BACK) dg = lu[h.x >= 0 ? hi16(h.x) : 0];
+#pragma unroll 1
+        for (int q = 0; q < steps; q++) {
+            const int2 rn = __ldg(ent);  // one step of padding follows the last
+            ent += G;
+            const int e0 = max(ea, 0), e1 = max(eb, 0);
+            const LT a0 = lu[lo16(e0)], b0 = x[hi16(e0)], a1 = lu[lo16(e1)], b1 = x[hi16(e1)];
+            if (ea >= 0) s -= a0 * b0;
+            if (eb >= 0) s2 += a1 * b1;
+            ea = rn.x;
+            eb = rn.y;
+        }
+        LT v = s - s2;
+        if constexpr (BACK) v *= dg;
+        if (h.x >= 0) *to = v;
+        if (h.w & 0x1000) {  // the level's last pass
+            gsync<G>(gm);
+            if constexpr (!BACK && G > 32) {
+                if (h.w & 0x2000) {  // split rows: their partials in order
+                    const int sb = __ldg(m.ssplit_ptr + L), se = __ldg(m.ssplit_ptr + L + 1);
+                    for (int k = sb + lane; k < se; k += G) {
+                        const int2 sp = __ldg(m.ssplit + k);
+                        const int first = lo16(sp.y), cnt = hi16(sp.y);
+                        LT t = x[sp.x];
+#pragma unroll 1
+                        for (int j = 0; j < cnt; j++) t += xp[first + j];
+                        x[sp.x] = t;
+                    }
+                    gsync<G>(gm);
+                }
+                L++;
+            }
+        }
+        h = hn;
+    }
+}
 
-// SP: pivots per round of the dense block's triangular solves (2 or 4)
-template <int G, typename LT, int SP>
+template <int G, int NPL, typename LT>
 __device__ void substitute(const DevMech &m, const CellPtr<LT> &c, int lane, unsigned gm) {
     LT *x = c.x;
     const LT *lu = c.lu;
@@ -1082,74 +1328,24 @@ __device__ void substitute(const DevMech &m, const CellPtr<LT> &c, int lane, uns
     // entries keep their value); split rows through partials (LU precision,
     // after the rate terms: free while solving)
     LT *xp = (LT *)(c.rs + m.R);
-    for (int L = 0; L < m.n_slev; L++) {
-        int b = __ldg(m.slev_ptr + L), e = __ldg(m.slev_ptr + L + 1);
-        for (int r = b + lane; r < e; r += G) {
-            const int2 job = __ldg(m.sjob + r);
-            const int i = lo16(job.y);
-            LT s = (G == 32 || i < m.n) ? x[i] : (LT)0, s2 = (LT)0;  // one-warp cells: no split rows
-            int qb = job.x, qe = job.x + hi16(job.y);
-            int q = qb;
-            for (; q + 1 < qe; q += 2) {
-                const int e2 = __ldg(m.sl_pack + q), e3 = __ldg(m.sl_pack + q + 1);
-                s -= lu[lo16(e2)] * x[hi16(e2)];
-                s2 += lu[lo16(e3)] * x[hi16(e3)];
-            }
-            if (q < qe) {
-                const int e2 = __ldg(m.sl_pack + q);
-                s -= lu[lo16(e2)] * x[hi16(e2)];
-            }
-            if (G == 32 || i < m.n) x[i] = s - s2;
-            else xp[i - m.n] = s - s2;
-        }
-        gsync<G>(gm);
-        if constexpr (G > 32) {
-            const int sb = __ldg(m.ssplit_ptr + L), se = __ldg(m.ssplit_ptr + L + 1);
-            if (se > sb) {
-                for (int k = sb + lane; k < se; k += G) {
-                    const int2 sp = __ldg(m.ssplit + k);
-                    const int first = lo16(sp.y), cnt = hi16(sp.y);
-                    LT t = x[sp.x];
-                    for (int j = 0; j < cnt; j++) t += xp[first + j];
-                    x[sp.x] = t;
-                }
-                gsync<G>(gm);
-            }
-        }
-    }
+    subst_passes<G, LT, false>(m, 0, m.n_fpass, lu, x, xp, lane, gm);
     const LT *A = lu + m.dbase;
     if (G <= 32 || lane < 32) {
         const unsigned wm = G <= 32 ? gm : 0xffffffffu;
-        switch ((m.D + 31) >> 5) {
-        case 0: break;
-        case 1: dense_subst<1, LT, SP>(A, m.D, m.LD, x + m.d, lane, wm); break;
-        case 2: dense_subst<2, LT, SP>(A, m.D, m.LD, x + m.d, lane, wm); break;
-        case 3: dense_subst<3, LT, SP>(A, m.D, m.LD, x + m.d, lane, wm); break;
-        default: dense_subst<4, LT, SP>(A, m.D, m.LD, x + m.d, lane, wm); break;
-        }
+        dense_rows<G * NPL>(m.D, [&](auto ns) { dense_subst<decltype(ns)::value>(A, m.D, m.LD, x + m.d, lane, wm); });
     }
     gsync<G>(gm);
     // backward, sparse rows by level
-    for (int L = 0; L < m.n_blev; L++) {
-        int b = __ldg(m.blev_ptr + L), e = __ldg(m.blev_ptr + L + 1);
-        for (int r = b + lane; r < e; r += G) {
-            int i = __ldg(m.brow + r);
-            LT s = x[i], s2 = (LT)0;
-            int qb = __ldg(m.su_ptr + i), qe = __ldg(m.su_ptr + i + 1);
-            int q = qb;
-            for (; q + 1 < qe; q += 2) {
-                const int e2 = __ldg(m.su_pack + q), e3 = __ldg(m.su_pack + q + 1);
-                s -= lu[lo16(e2)] * x[hi16(e2)];
-                s2 += lu[lo16(e3)] * x[hi16(e3)];
-            }
-            if (q < qe) {
-                const int e2 = __ldg(m.su_pack + q);
-                s -= lu[lo16(e2)] * x[hi16(e2)];
-            }
-            x[i] = (s - s2) * lu[__ldg(m.udiag + i)];
-        }
-        gsync<G>(gm);
-    }
+    subst_passes<G, LT, true>(m, m.n_fpass, m.n_fpass + m.n_bpass, lu, x, xp, lane, gm);
+}
+
+// J at the state in ys and the factorisation of I - gamma J, out of line;
+// returns true if every pivot is usable
+template <int G, int NPL, typename LT, bool W>
+__device__ __noinline__ bool setup_matrix(const DevMech &m, int base, double gamma, int lane, unsigned gm) {
+    const CellPtr<LT> c(base, m);
+    assemble<G, LT, W>(m, c, gamma, lane, gm, 0, nullptr);
+    return factor<G, NPL, LT>(m, c, lane, gm);
 }
 
 template <int G, int NPL>
@@ -1220,8 +1416,8 @@ __device__ __forceinline__ float ctl_powf(float x, float p) {
 // Newton-Raphson step w <- w (2 - d w) in FP64; outside the FP32 normal
 // range a division
 __device__ __forceinline__ double recip_refined(double d) {
-    if (d > 1e-37 && d < 1e37) {
-        const double w = (double)__frcp_rn((float)d);
+    if (pos_gt(d, 1e-37) && __double_as_longlong(d) < __double_as_longlong(1e37)) {
+        const double w = widen(__frcp_rn(narrow(d)));
         return w * fma(-d, w, 2.0);
     }
     return 1.0 / d;
@@ -1282,6 +1478,10 @@ __device__ int integrate_cell(const DevMech &m, const CellPtr<LT> &c, double *__
                               CellStats &st, double *__restrict__ y_copy = nullptr) {
     const int n = m.n;
     constexpr bool EXACT = sizeof(LT) == 8;  // the plain FP64 form
+    // whether z1 / l1 is rounded before the Newton residual takes it or fused
+    // into its sum: fixed per shape, so that a build's choice of contractions
+    // cannot move a cell's step sequence
+    constexpr bool ROUND_Z1 = G == 32 && !W && (EXACT || NPL <= 3);
     using C = Ctl<EXACT>;
     const double h_in = step_io ? *step_io : 0.0;
     st.steps = st.newton = st.jac = st.errfail = st.ordsum = 0;
@@ -1290,6 +1490,7 @@ __device__ int integrate_cell(const DevMech &m, const CellPtr<LT> &c, double *__
     bool bad = false;
     for (int i = lane; i < m.n_env; i += G) bad |= !finite_bits(env_cell[i]);
     double z[QMAX + 1][NPL], e[NPL], ep[NPL], w[NPL], f[NPL];
+    LT wn[NPL];  // the weights as the Newton update's norm takes them
 #pragma unroll
     for (int s = 0; s < NPL; s++) {
         int p = lane + G * s;
@@ -1308,6 +1509,7 @@ __device__ int integrate_cell(const DevMech &m, const CellPtr<LT> &c, double *__
     };
     if (gany<G>(bad, gm)) return fail_early(ST_NONFINITE);
 
+#pragma unroll 1
     for (int k = lane; k < m.R; k += G) {
         double a, b;
         rate_constant(m, k, env_cell, a, b);
@@ -1326,6 +1528,7 @@ __device__ int integrate_cell(const DevMech &m, const CellPtr<LT> &c, double *__
             double a = 1.0;
             if (p < n) a = atol_len == 1 ? __ldg(atol) : __ldg(atol + __ldg(m.perm + p));
             w[s] = (p < n) ? C::weight(rtol, z[0][s], a) : 0.0;
+            wn[s] = norm_weight<LT>(w[s]);
         }
     };
     auto any_nonfinite = [&](const double(&v)[NPL]) {
@@ -1367,7 +1570,13 @@ __device__ int integrate_cell(const DevMech &m, const CellPtr<LT> &c, double *__
     int q = 1, qwait = 2, nst = 0, nst_lu = 0;
     double h_held = h;
     bool have_lu = false, need_setup = true, ep_valid = false;
-    double t = 0.0, gamma_lu = 0.0, rgamma_lu = 0.0;
+    double t = 0.0, gamma_lu = 0.0;
+    // gamma, its drift from the factored one beyond the limit and the
+    // update's scaling are functions of (h, q, gamma_lu): kept, and formed
+    // again only after one of them changed (`moved`)
+    double gamma = 0.0, rl1 = 0.0;
+    LT scale = (LT)1;
+    bool moved = true, drifted = false;
     int status = ST_OK;
     // The mixed form takes the controller's tests on squared norms (the same
     // decisions as comparing the norms themselves, without roots): Newton
@@ -1378,41 +1587,53 @@ __device__ int integrate_cell(const DevMech &m, const CellPtr<LT> &c, double *__
     constexpr double NEWTON_TOL2 = NEWTON_TOL * NEWTON_TOL;
     constexpr double RHO_DIV2 = RHO_DIV * RHO_DIV;
 
-    while (t < T) {
+    while (pos_gt(T, t)) {
         if (nst >= max_steps) { status = ST_MAXSTEPS; break; }
         set_weights();
         int nef = 0, ncf = 0;
         bool last = false;
-        double err2 = 0.0;
+        double err2 = 0.0, t_new = 0.0;
         bool accepted = false;
         while (!accepted) {
             last = false;
             h_held = h;
-            if (t + h >= T) {
-                if (t + h > T) {
+            t_new = t + h;
+            if (pos_ge(t_new, T)) {
+                if (pos_gt(t_new, T)) {
                     double eta = (T - t) / h;
                     nord_rescale<NPL>(z, q, eta);
                     h = T - t;
+                    moved = true;
                 }
                 last = true;
+                t_new = T;
             }
             nord_predict<NPL>(z, q);
-            const double rl1 = m.inv_l1[q];
-            const double gamma = C::ratio(h, m.lcoef[q][1], rl1);
+            if (moved) {
+                rl1 = m.inv_l1[q];
+                gamma = C::ratio(h, m.lcoef[q][1], rl1);
+                drifted = false;
+                scale = (LT)1;
+                if (have_lu && __double_as_longlong(gamma) != __double_as_longlong(gamma_lu)) {
+                    const double gr = C::ratio(gamma, gamma_lu, 1.0 / gamma_lu);
+                    drifted = fabs(gr - 1.0) > DGMAX;
+                    scale = (LT)2 / ((LT)1 + to_lu<LT>(gr));
+                }
+                moved = false;
+            }
             bool jcur = false, lu_fail = false;
-            if (!have_lu || need_setup || nst >= nst_lu + MSBJ ||
-                fabs(C::ratio(gamma, gamma_lu, rgamma_lu) - 1.0) > DGMAX) {
+            if (!have_lu || need_setup || nst >= nst_lu + MSBJ || drifted) {
 #pragma unroll
                 for (int s = 0; s < NPL; s++) {
                     int p = lane + G * s;
                     if (p < n) c.ys[p] = z[0][s];
                 }
                 gsync<G>(gm);
-                assemble<G, LT, W>(m, c, gamma, lane, gm, 0, nullptr);
-                lu_fail = !factor<G, LT>(m, c, lane, gm);
+                lu_fail = !setup_matrix<G, NPL, LT, W>(m, c.base, gamma, lane, gm);
                 st.jac++;
                 gamma_lu = gamma;
-                rgamma_lu = 1.0 / gamma;
+                drifted = false;
+                scale = (LT)1;
                 nst_lu = nst;
                 have_lu = !lu_fail;
                 need_setup = false;
@@ -1424,19 +1645,19 @@ __device__ int integrate_cell(const DevMech &m, const CellPtr<LT> &c, double *__
                 LT dprev2 = (LT)0;
 #pragma unroll
                 for (int s = 0; s < NPL; s++) e[s] = 0.0;
-                const LT scale = (gamma != gamma_lu)
-                                     ? (LT)2 / ((LT)1 + to_lu<LT>(C::ratio(gamma, gamma_lu, rgamma_lu)))
-                                     : (LT)1;
-                for (int it = 0; it < NEWTON_MAXIT; it++) {
-                    eval_f_at<G, NPL, LT, W>(m, c, z[0], 1.0, e, f, lane, gm);
+#pragma unroll 1
+                for (int it = 0; it < NEWTON_MAXIT; it++) {  // one copy of the loop's code (instruction cache)
+                    eval_f_newton<G, NPL, LT, W>(m, c, z[0], e, it == 0, f, lane, gm);
                     st.newton++;
                     if (any_nonfinite(f)) break;
 #pragma unroll
                     for (int s = 0; s < NPL; s++) {
                         int p = lane + G * s;
-                        if (p < n) c.x[p] = to_lu<LT>(-(e[s] - gamma * f[s] + z[1][s] * rl1));
+                        const double r0 = fma(-gamma, f[s], e[s]);
+                        const double r = ROUND_Z1 ? __dadd_rn(r0, __dmul_rn(z[1][s], rl1)) : fma(z[1][s], rl1, r0);
+                        if (p < n) c.x[p] = to_lu<LT>(-r);
                     }
-                    substitute<G, LT, subst_pivots<G, NPL, LT>()>(m, c, lane, gm);
+                    substitute<G, NPL, LT>(m, c, lane, gm);
                     // the update's norm in the LU precision (it only steers the iteration)
                     LT dsq = (LT)0;
                     bool nf = false;
@@ -1445,8 +1666,9 @@ __device__ int integrate_cell(const DevMech &m, const CellPtr<LT> &c, double *__
                         int p = lane + G * s;
                         LT xl = (p < n) ? c.x[p] : (LT)0;
                         xl *= scale;
-                        e[s] += from_lu(xl);
-                        dsq += upd_term(xl, w[s]);
+                        if (it == 0) e[s] = from_lu(xl);  // e was zero
+                        else e[s] += from_lu(xl);
+                        dsq += upd_term(xl, wn[s]);
                         nf |= !isfinite(xl);
                     }
                     // EXACT: the norm itself, as the oracle tests it; mixed:
@@ -1469,6 +1691,7 @@ __device__ int integrate_cell(const DevMech &m, const CellPtr<LT> &c, double *__
                 if (!jcur) { need_setup = true; continue; }
                 if (++ncf >= MAX_NCF) { status = lu_fail ? ST_SINGULAR : ST_NEWTON; break; }
                 h *= ETA_CF;
+                moved = true;
                 if (h < hmin) { status = ST_ERRTEST; break; }
                 nord_rescale<NPL>(z, q, ETA_CF);
                 need_setup = true;
@@ -1481,9 +1704,10 @@ __device__ int integrate_cell(const DevMech &m, const CellPtr<LT> &c, double *__
                 for (int s = 0; s < NPL; s++) { double a = e[s] * w[s]; es += a * a; }
                 err2 = C::norm(m.ecoef[q], m.ecoef2[q], gsum<G>(es, gm), n, m.rn);
             }
-            if (err2 > 1.0) {
+            if (pos_gt(err2, 1.0)) {
                 nord_retract<NPL>(z, q);
                 st.errfail++;
+                moved = true;
                 if (++nef >= MAX_NEF) { status = ST_ERRTEST; break; }
                 if (nef >= 3) {
                     h *= 0.1;
@@ -1515,12 +1739,12 @@ __device__ int integrate_cell(const DevMech &m, const CellPtr<LT> &c, double *__
                 for (int s = 0; s < NPL; s++) z[j][s] += lj * e[s];
             }
         }
-        t = last ? T : t + h;
+        t = t_new;
         nst++;
         st.ordsum += q;
         if (any_nonfinite(z[0])) { status = ST_NONFINITE; break; }
 
-        if (--qwait <= 0 && t < T) {
+        if (--qwait <= 0 && !last) {
             // eta = 1 / ((c err)^(1/(p+1)) + 1e-6), from the squared norms
             double eta_q = C::eta(1.2, err2, q + 1);
             double eta_m = 0.0, eta_p = 0.0;
@@ -1564,6 +1788,7 @@ __device__ int integrate_cell(const DevMech &m, const CellPtr<LT> &c, double *__
                 }
                 q = qn;
                 h *= eta;
+                moved = true;
                 nord_rescale<NPL>(z, q, eta);
                 qwait = q + 1;
             }

@@ -6,8 +6,15 @@
 // the compiler (position p holds species perm[p]); only the state/env/atol
 // loads and stores translate back to declaration order.
 #pragma once
+#include <stddef.h>
 #include <stdint.h>
 #include <vector_types.h>
+
+#ifdef __CUDACC__
+#define CAMP_HD __host__ __device__
+#else
+#define CAMP_HD
+#endif
 
 #define CAMP_QMAX 5
 #define CAMP_MAXFAC 3  // at most 3 factors (with multiplicity) per rate term
@@ -55,8 +62,53 @@ inline int camp_alt_lanes(int n) {
 #define CAMP_OP_DIV 0x80000000u
 #define CAMP_OP_TGT(op) ((int)((op)&0xFFFFu))
 #define CAMP_OP_SRC(op) ((int)(((op) >> 16) & 0x7FFFu))
+#define CAMP_OP_NOSRC 0x7FFF  // no source: with DIV no op, without it a pivot's reciprocal
+
+// Dynamic shared memory one block may use (227 KB less room for a block
+// group's static reduction scratch).
+constexpr int CAMP_MAX_SMEM = 227 * 1024 - 256;
+
+// Shared-memory layout of one cell (byte offsets).  rs holds the R rate
+// terms, then n_part partial sums (of split forcing sums inside an f
+// evaluation, of split substitution and factorisation rows inside a solve);
+// pw the water parameter's per-cell values (n_pw doubles, and n_pw64 more in
+// the FP64 form; none without one); fb the odd halves of the
+// forcing sums (n + n_fpart doubles), which saves FP64 adds where a lane owns
+// few positions: one-warp cells and block cells of up to 4 positions a lane.
+// Other cells, and a cell that only fits without it, have none (fb = -1) and
+// add the two halves of a sum where the sum ends.
+struct CellSmem {
+    int ys, rs, kf, kr, pw, x, lu, fb, bytes;
+};
+CAMP_HD inline int camp_align16(int b) { return (b + 15) & ~15; }
+CAMP_HD inline CellSmem cell_smem(int n, int R, int n_rev, int nlu, int lu_elem, int n_part, int n_fpart, int n_pw,
+                                  int n_pw64, int lanes) {
+    CellSmem c;
+    int o = 0;
+    c.ys = o; o = camp_align16(o + 8 * n);
+    c.rs = o; o = camp_align16(o + 8 * (R + n_part));
+    c.kf = o; o = camp_align16(o + 8 * R);
+    c.kr = o; o = camp_align16(o + 8 * n_rev);
+    c.pw = o; o = camp_align16(o + 8 * (n_pw + (lu_elem == 8 ? n_pw64 : 0)));
+    // the substitution vector shares the rate-term scratch when it fits:
+    // the rate terms live only inside one f evaluation, the vector only
+    // inside one Newton solve, and the Jacobian assembly keeps its FP32
+    // copy of y in ys instead
+    if (8 * R >= lu_elem * n) {
+        c.x = c.rs;
+    } else {
+        c.x = o;
+        o = camp_align16(o + lu_elem * n);
+    }
+    c.lu = o; o = camp_align16(o + lu_elem * nlu);
+    const int with = camp_align16(o + 8 * (n + n_fpart));
+    c.fb = with <= CAMP_MAX_SMEM && n <= (lanes == 32 ? 8 : 4) * lanes ? o : -1;
+    c.bytes = c.fb >= 0 ? with : o;
+    return c;
+}
 
 struct DevMech {
+    CellSmem smem4, smem8;  // shared memory of one cell, FP32 and FP64 LU
     int n;            // species
     int R;            // process instances
     int n_env;
@@ -77,16 +129,18 @@ struct DevMech {
     // w = rev2 (positions; 16-bit fields, 0xffff = none; rv = kr index)
     const int4 *rpack;    // [R]
 
-    // --- forcing gather f_p = sum_q c_q r_k(q), as lane jobs ---
-    // entry q: process | index into fcoef << 16
-    const int *fpk;       // [nf]
-    const double *fcoef;  // the mechanism's distinct net coefficients
-    // lane l's jobs: flane_ptr[l] .. flane_ptr[l+1], balanced by entry count.
-    // Job: x = first entry, y = destination | entry count << 16; a destination
-    // d < n is the position's f, d >= n the partial sum d - n of a position
-    // whose sum was split into chunks (block cells only)
-    const int *flane_ptr; // [lanes+1]
-    const int2 *fjob;
+    // --- forcing gather f_p = sum_q c_q r_k(q), as one flat list per lane ---
+    // step * lanes + lane, n_gstep steps (two more of padding follow for the
+    // read-ahead).  gth: x = a pair of entries of the lane's current sum, their
+    // processes in 15 bits each (low half: to the sum's even accumulator, high
+    // half: to its odd one; 0x8000 in a half: no entry), y = the sum's
+    // destination at its last pair, else -1; gcf: the pair's coefficients.  A
+    // destination d < n is the position's f, d >= n the partial sum d - n of a
+    // position whose sum was split into chunks (block cells only).
+    const int2 *gth;
+    const double2 *gcf;
+    int n_gstep;
+    int n_fpart;          // partial sums of split forcing sums
     int n_part;           // partial sums of split forcing sums, substitution
                           // rows and factorisation rows (scratch after the
                           // rate terms; counted in FP64 values)
@@ -96,69 +150,65 @@ struct DevMech {
 
     // --- Jacobian, assembled straight into I - gamma J ---
     int nnzJ;
-    // FP32: per-lane flat entry lists (nonzeros spread over the lanes by
-    // entry count).  Record: x = bits of the FP32 coefficient, y = k (signed
-    // 16 bits; -(r+1) for a reverse constant) | o1 << 16, z = LU offset |
-    // diag << 16 | last-entry-of-nonzero << 17, w = o2 | CSR index << 16
-    const int *jl_ptr;    // [lanes+1]
-    const int4 *jl_rec;   // [entries + empty non-zeros]
-    // FP64: by non-zero t: x = first entry, y = end entry, z = LU offset,
-    // w = diagonal; entry q: constant jk (k, or -(r+1) for a reverse constant),
-    // other factors jo (positions, -1 = none), coefficient jc
-    const int4 *jnz;      // [nnzJ]
-    const int *jk;        // [nj]
-    const int *jo;        // [nj][2]
-    const double *jc;     // [nj]
+    // Per-lane flat entry lists (nonzeros spread over the lanes by entry
+    // count), jls[step * lanes + lane].  Record: x = bits of the FP32
+    // coefficient, y = k (signed 16 bits; -(r+1) for a reverse constant) |
+    // o1 << 16 (0xffff: none), z = LU offset | diag << 16 | last entry of the
+    // nonzero << 17, w = o2 | CSR index << 16; jlc: the coefficients in FP64.
+    // The last record of a lane's list has bit 18 of z set; warp w of the cell
+    // has lists of at most n_jstep[w].
+    const int4 *jls;
+    const double *jlc;
+    int n_jstep[8];
 
     // --- LU storage: sparse rows [0, nsp) then a dense trailing block ---
     int nlu;              // storage entries
     int d;                // first position of the dense block (= n when there is none)
     int D;                // dense block size n - d
-    int LD;               // dense block row stride (odd, to spread shared-memory banks)
+    int LD;           // dense block row stride, 4 mod 8
     int dbase;            // storage offset of the dense block
 
-    // factorisation of the sparse part: row-wise (up-looking) ops as lane
-    // jobs, by level.  Op: DIV flag | source << 16 | target (LU offsets; a
-    // division makes the multiplier, an update subtracts it times the
-    // source).  Job: x = first op in lops, y = op count | partial slots << 16,
-    // z = row | (1 << 16 if the job ends by taking the row's pivot
-    // reciprocal), w = partial base.  An update whose target has bit 15 set
-    // adds to partial w + (target & 0x7fff) instead of the LU value.  Per
-    // level, the rows cut into chunks then get a reduction (x = row |
-    // reciprocal flag << 16, y = first entry of lred_off, z = shared columns
-    // ns | chunks << 16, w = partial base; chunk c's slot s is w + c ns + s)
-    // and their tail ops (x = first op, y = count).
+    // factorisation of the sparse part: row-wise (up-looking) ops, level by
+    // level as one list per lane, fst[step * lanes + lane] for the steps
+    // fst_ptr[L] .. fst_ptr[L+1] of level L (one padding step follows the
+    // last).  Op: DIV flag | source << 16 | target (LU offsets; a division
+    // makes the multiplier, an update subtracts it times the source); with
+    // the source CAMP_OP_NOSRC it takes the reciprocal of its target (a
+    // row's pivot) or, with the DIV flag, does nothing.  An update whose
+    // target has bit 15 set adds to a partial sum instead of an LU value (the
+    // level's fst_part[L] partials start at zero).  Per level, the rows cut
+    // into chunks then get a reduction (x = row | reciprocal flag << 16, y =
+    // first entry of lred_off, z = shared columns ns | chunks << 16, w =
+    // partial base; chunk c's slot s is w + c ns + s) and their tail ops (x =
+    // first op in lops, y = count).
     int n_flev;
-    const int *ljob_ptr;  // [n_flev+1] into ljob
-    const int4 *ljob;
+    const int *fst_ptr;   // [n_flev+1]
+    const int *fst_part;  // [n_flev]
+    const uint32_t *fst;
     const uint32_t *lops;
     const int *lred_ptr;  // [n_flev+1] into lred / ltail
     const int4 *lred;
     const int *lred_off;  // LU offsets of the shared columns
     const int2 *ltail;
 
-    // substitution entries: LU offset | column << 16
-    const int *sl_pack;   // L entries of the sparse rows, row by row
-    const int *su_pack;   // U entries of the sparse rows, row by row
-
-    // forward substitution of the sparse part: lane jobs by level (jobs
-    // within a level ordered to balance the lanes) over the rows that have L
-    // entries.  Job: x = first entry of sl_pack, y = destination | entry count
-    // << 16; a destination d < n is row d, finished by the job, d >= n the
-    // partial dot product d - n of a row cut into chunks; the level's split
-    // rows (x = row, y = first partial | chunk count << 16) then subtract
-    // their partials in order.
-    int n_slev;
-    const int *slev_ptr;  // [n_slev+1] into sjob
-    const int2 *sjob;
-    const int *ssplit_ptr; // [n_slev+1] into ssplit
+    // Substitution of the sparse part, as passes over the lanes: in pass p
+    // lane l takes the record sub_pass[p * lanes + l]: x = its row (-1: none),
+    // y, z = the first two entries (LU offset | column << 16, -1: none), w =
+    // entry pairs of the pass | 0x1000 on its level's last pass | 0x2000 if
+    // that level has split rows | first step in `sub` << 14; sub[step * lanes
+    // + l] holds the pairs from the second on.  One padding pass and step
+    // follow the last.  The first n_fpass passes are the forward substitution
+    // of the rows that have L entries, level by level; a row number >= n is
+    // the partial dot product (row - n) of a row cut into chunks, and level
+    // L's split rows (ssplit_ptr[L] ..: x = row, y = first partial | chunk
+    // count << 16) then subtract their partials in order.  The n_bpass passes
+    // after them are the backward substitution of the sparse rows (i < d), row
+    // | LU offset of its reciprocal pivot << 16 in x.
+    const int4 *sub_pass;
+    const int2 *sub;
+    int n_fpass, n_bpass;
+    const int *ssplit_ptr;
     const int2 *ssplit;
-
-    // backward substitution of the sparse rows (i < d), by level
-    int n_blev;
-    const int *blev_ptr;  // [n_blev+1] into brow
-    const int *brow;
-    const int *su_ptr;    // [n+1] into su_pack
     const int *udiag;     // [n] storage offset of U(i,i) for sparse rows
 
     const int *perm;      // [n] position -> species (declaration order)

@@ -33,12 +33,10 @@ __device__ __forceinline__ unsigned group_mask() {
 template <int G, int NPL, typename LT, bool W>
 __global__ void __maxnreg__((G == 64 && NPL == 4) || (G == 128 && sizeof(LT) == 8) ? 168
                             : ((sizeof(LT) == 8 || G > 32) ? 255 : (NPL >= 6 ? 224 : 168)))
-    k_solve(DevMech m, SolveArgs a) {
-    extern __shared__ __align__(16) char smem[];
+    k_solve(const __grid_constant__ DevMech m, const __grid_constant__ SolveArgs a) {
     const int group = threadIdx.x / G, lane = threadIdx.x % G;
     const unsigned gm = group_mask<G>();
-    const CellSmem L = cell_smem(m.n, m.R, m.n_rev, m.nlu, (int)sizeof(LT), m.n_part, m.n_pw, m.n_pw64);
-    CellPtr<LT> c(smem + group * L.bytes, m);
+    const CellPtr<LT> c(group * CellPtr<LT>::layout(m).bytes, m);
     long long cell = a.queue ? 0 : (long long)blockIdx.x * a.cpb + group;
     for (;;) {
         if (a.queue) {
@@ -90,7 +88,7 @@ __global__ void __maxnreg__((G == 64 && NPL == 4) || (G == 128 && sizeof(LT) == 
 
 // Rate constants of every process of every cell, [cell][R] in process order.
 template <int G>
-__global__ void k_rates(DevMech m, long long n_cells, const double *env, double *kf, double *kr) {
+__global__ void k_rates(const __grid_constant__ DevMech m, long long n_cells, const double *env, double *kf, double *kr) {
     const long long cell = (long long)blockIdx.x * (blockDim.x / G) + threadIdx.x / G;
     const int lane = threadIdx.x % G;
     if (cell >= n_cells) return;
@@ -124,15 +122,13 @@ __device__ __forceinline__ void load_cell(const DevMech &m, const CellPtr<LT> &c
 
 // f(y) of every cell, [cell][n] in declaration order.
 template <int G, int NPL, typename LT, bool W>
-__global__ void k_forcing(DevMech m, long long n_cells, const double *state, const double *env,
+__global__ void k_forcing(const __grid_constant__ DevMech m, long long n_cells, const double *state, const double *env,
                           double *f_out) {
-    extern __shared__ __align__(16) char smem[];
     const int group = threadIdx.x / G, lane = threadIdx.x % G;
     const unsigned gm = group_mask<G>();
     const long long cell = (long long)blockIdx.x * (blockDim.x / G) + group;
     if (cell >= n_cells) return;
-    const CellSmem L = cell_smem(m.n, m.R, m.n_rev, m.nlu, (int)sizeof(LT), m.n_part, m.n_pw, m.n_pw64);
-    CellPtr<LT> c(smem + group * L.bytes, m);
+    const CellPtr<LT> c(group * CellPtr<LT>::layout(m).bytes, m);
     double y[NPL], f[NPL];
     load_cell<G, NPL, LT, W>(m, c, state + cell * m.n, env + cell * m.n_env, y, lane, gm);
     eval_f<G, NPL, LT, W>(m, c, y, f, lane, gm);
@@ -146,15 +142,13 @@ __global__ void k_forcing(DevMech m, long long n_cells, const double *state, con
 // Jacobian values of every cell, [cell][nnzJ] in species-CSR order, computed
 // in precision LT (the assembly precision of the corresponding solve form).
 template <int G, int NPL, typename LT, bool W>
-__global__ void k_jacobian(DevMech m, long long n_cells, const double *state, const double *env,
+__global__ void k_jacobian(const __grid_constant__ DevMech m, long long n_cells, const double *state, const double *env,
                            double *jac) {
-    extern __shared__ __align__(16) char smem[];
     const int group = threadIdx.x / G, lane = threadIdx.x % G;
     const unsigned gm = group_mask<G>();
     const long long cell = (long long)blockIdx.x * (blockDim.x / G) + group;
     if (cell >= n_cells) return;
-    const CellSmem L = cell_smem(m.n, m.R, m.n_rev, m.nlu, (int)sizeof(LT), m.n_part, m.n_pw, m.n_pw64);
-    CellPtr<LT> c(smem + group * L.bytes, m);
+    const CellPtr<LT> c(group * CellPtr<LT>::layout(m).bytes, m);
     double y[NPL];
     load_cell<G, NPL, LT, W>(m, c, state + cell * m.n, env + cell * m.n_env, y, lane, gm);
     assemble<G, LT, W>(m, c, 0.0, lane, gm, 1, jac + cell * (long long)m.nnzJ);
@@ -164,23 +158,20 @@ __global__ void k_jacobian(DevMech m, long long n_cells, const double *state, co
 // precision LT; b and x [cell][n] in declaration order; status 4 on a
 // tiny pivot (x then left unwritten).
 template <int G, int NPL, typename LT, bool W>
-__global__ void k_lu_solve(DevMech m, long long n_cells, const double *state, const double *env,
+__global__ void k_lu_solve(const __grid_constant__ DevMech m, long long n_cells, const double *state, const double *env,
                            double gamma, const double *b, double *x, int *status) {
-    extern __shared__ __align__(16) char smem[];
     const int group = threadIdx.x / G, lane = threadIdx.x % G;
     const unsigned gm = group_mask<G>();
     const long long cell = (long long)blockIdx.x * (blockDim.x / G) + group;
     if (cell >= n_cells) return;
-    const CellSmem L = cell_smem(m.n, m.R, m.n_rev, m.nlu, (int)sizeof(LT), m.n_part, m.n_pw, m.n_pw64);
-    CellPtr<LT> c(smem + group * L.bytes, m);
+    const CellPtr<LT> c(group * CellPtr<LT>::layout(m).bytes, m);
     double y[NPL];
     load_cell<G, NPL, LT, W>(m, c, state + cell * m.n, env + cell * m.n_env, y, lane, gm);
-    assemble<G, LT, W>(m, c, gamma, lane, gm, 0, nullptr);
-    bool ok = factor<G, LT>(m, c, lane, gm);
+    const bool ok = setup_matrix<G, NPL, LT, W>(m, c.base, gamma, lane, gm);
     if (lane == 0) status[cell] = ok ? 0 : ST_SINGULAR;
     if (!ok) return;
     for (int p = lane; p < m.n; p += G) c.x[p] = (LT)b[cell * m.n + __ldg(m.perm + p)];
-    substitute<G, LT, subst_pivots<G, NPL, LT>()>(m, c, lane, gm);
+    substitute<G, NPL, LT>(m, c, lane, gm);
     for (int p = lane; p < m.n; p += G) x[cell * m.n + __ldg(m.perm + p)] = (double)c.x[p];
 }
 

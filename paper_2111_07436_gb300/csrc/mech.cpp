@@ -292,37 +292,41 @@ static void pack_records(HostMech &h) {
             o[3] |= ((p.slot + 1) | (p.la << 11) | (p.lb << 13)) << 16;
         }
     }
-    // gather entries as 4 bytes each: process | index into the table of the
-    // mechanism's distinct coefficients << 16
-    h.fcoef.clear();
-    h.fpk.assign(h.fk.size(), 0);
+    // the lanes' sums as one flat list of entry pairs per lane (DevMech::gth)
     {
-        std::unordered_map<uint64_t, int> seen;
-        for (size_t q = 0; q < h.fk.size(); q++) {
-            uint64_t bits;
-            std::memcpy(&bits, &h.fc[q], 8);
-            auto it = seen.find(bits);
-            int ci;
-            if (it == seen.end()) {
-                ci = (int)h.fcoef.size();
-                seen.emplace(bits, ci);
-                h.fcoef.push_back(h.fc[q]);
-            } else {
-                ci = it->second;
+        const int NL = h.lanes;
+        if (R > 0x7fff) throw std::runtime_error("forcing table does not fit 15-bit fields");
+        auto pairs = [&](int i) { return std::max(1, (((int)((unsigned)h.fjob[2 * i + 1] >> 16)) + 1) / 2); };
+        h.n_gstep = 0;
+        for (int l = 0; l < NL; l++) {
+            int steps = 0;
+            for (int i = h.flane_ptr[l]; i < h.flane_ptr[l + 1]; i++) steps += pairs(i);
+            h.n_gstep = std::max(h.n_gstep, steps);
+        }
+        const size_t cells = (size_t)(h.n_gstep + 2) * NL;
+        h.gth.assign(cells * 2, -1);
+        for (size_t q = 0; q < cells; q++) h.gth[2 * q] = (int)0x80008000u;
+        h.gcf.assign(cells * 2, 0.0);
+        for (int l = 0; l < NL; l++) {
+            size_t q = l;
+            for (int i = h.flane_ptr[l]; i < h.flane_ptr[l + 1]; i++) {
+                const int first = h.fjob[2 * i], dst = h.fjob[2 * i + 1] & 0xffff;
+                const int cnt = (int)((unsigned)h.fjob[2 * i + 1] >> 16), np = pairs(i);
+                for (int t = 0; t < np; t++, q += NL) {
+                    unsigned w = 0;
+                    for (int e = 0; e < 2; e++) {
+                        if (2 * t + e >= cnt) { w |= 0x8000u << (16 * e); continue; }
+                        w |= (unsigned)h.fk[first + 2 * t + e] << (16 * e);
+                        h.gcf[2 * q + e] = h.fc[first + 2 * t + e];
+                    }
+                    h.gth[2 * q] = (int)w;
+                    if (t == np - 1) h.gth[2 * q + 1] = dst;
+                }
             }
-            if (h.fk[q] > 0xffff || ci > 0xffff) throw std::runtime_error("forcing table does not fit 16-bit fields");
-            h.fpk[q] = h.fk[q] | (ci << 16);
         }
     }
 
     const int nnzJ = (int)h.colidx.size();
-    h.jnz.assign((size_t)nnzJ * 4, 0);
-    for (int t = 0; t < nnzJ; t++) {
-        h.jnz[(size_t)t * 4 + 0] = h.jptr[t];
-        h.jnz[(size_t)t * 4 + 1] = h.jptr[t + 1];
-        h.jnz[(size_t)t * 4 + 2] = h.jdst[t];
-        h.jnz[(size_t)t * 4 + 3] = h.jdiag[t];
-    }
     // per-lane flat Jacobian entry lists, longest-processing-time over the lanes
     {
         const int NL = h.lanes;
@@ -340,32 +344,41 @@ static void pack_records(HostMech &h) {
             load[best] += cnt(t);
         }
         if (nnzJ > 65535) throw std::runtime_error("too many Jacobian non-zeros for the packed records");
-        h.jl_ptr.assign(1, 0);
-        h.jl_rec.clear();
-        auto emit = [&](float c, int k, int o1, int o2, int t, bool last) {
-            int cb;
-            std::memcpy(&cb, &c, 4);
-            h.jl_rec.push_back(cb);
-            h.jl_rec.push_back((k & 0xffff) | (field16(o1) << 16));
-            h.jl_rec.push_back(h.jdst[t] | (h.jdiag[t] << 16) | ((last ? 1 : 0) << 17));
-            h.jl_rec.push_back(field16(o2) | (t << 16));
-        };
-        for (auto &v : lanes) {
-            for (int t : v) {
+        // the longest lists on the first lanes, so that they share a warp
+        std::vector<int> by(NL);
+        for (int l = 0; l < NL; l++) by[l] = l;
+        std::stable_sort(by.begin(), by.end(), [&](int a, int b) { return load[a] > load[b]; });
+        const size_t cells = (size_t)std::max(1, load[by[0]]) * NL;
+        for (int w = 0; w < 8; w++) h.n_jstep[w] = 32 * w < NL ? std::max(1, load[by[32 * w]]) : 0;
+        h.jls.assign(cells * 4, 0);
+        h.jlc.assign(cells, 0.0);
+        for (size_t q = 0; q < cells; q++) {
+            h.jls[4 * q + 1] = (int)0xffff0000u;
+            h.jls[4 * q + 2] = 1 << 18;
+            h.jls[4 * q + 3] = 0xffff;
+        }
+        for (int l = 0; l < NL; l++) {
+            int step = 0;
+            auto emit = [&](double c, int k, int o1, int o2, int t, bool last) {
+                const size_t q = (size_t)step++ * NL + l;
+                const float cf = (float)c;
+                std::memcpy(&h.jls[4 * q], &cf, 4);
+                h.jls[4 * q + 1] = (k & 0xffff) | (field16(o1) << 16);
+                h.jls[4 * q + 2] = h.jdst[t] | (h.jdiag[t] << 16) | ((last ? 1 : 0) << 17) |
+                                   ((step == load[by[l]] ? 1 : 0) << 18);
+                h.jls[4 * q + 3] = field16(o2) | (t << 16);
+                h.jlc[q] = c;
+            };
+            for (int t : lanes[by[l]]) {
                 int b = h.jptr[t], e = h.jptr[t + 1];
-                if (b == e) emit(0.0f, 0, -1, -1, t, true);
+                if (b == e) emit(0.0, 0, -1, -1, t, true);
                 for (int q = b; q < e; q++) {
                     if (h.jk[q] < -32768 || h.jk[q] > 32767) throw std::runtime_error("process index too large");
-                    emit((float)h.jc[q], h.jk[q], h.jo[2 * q], h.jo[2 * q + 1], t, q == e - 1);
+                    emit(h.jc[q], h.jk[q], h.jo[2 * q], h.jo[2 * q + 1], t, q == e - 1);
                 }
             }
-            h.jl_ptr.push_back((int)h.jl_rec.size() / 4);
         }
     }
-    h.sl_pack.resize(h.sl_off.size());
-    for (size_t q = 0; q < h.sl_off.size(); q++) h.sl_pack[q] = field16(h.sl_off[q]) | (field16(h.sl_col[q]) << 16);
-    h.su_pack.resize(h.su_off.size());
-    for (size_t q = 0; q < h.su_off.size(); q++) h.su_pack[q] = field16(h.su_off[q]) | (field16(h.su_col[q]) << 16);
 }
 
 static void build_structure(HostMech &h) {
@@ -551,10 +564,13 @@ static RowSplit split_row(const std::vector<uint32_t> &ops, int CH) {
 // a longer chunk length is taken when the level's splits would need more.
 static const long long kLevelPartials = 2048;
 
+static const uint32_t kFactorNop = CAMP_OP_DIV | ((uint32_t)CAMP_OP_NOSRC << 16);
+
 static void build_factor_jobs(HostMech &h) {
     const int NL = h.lanes;
-    h.ljob_ptr.assign(1, 0);
-    h.ljob.clear();
+    h.fst_ptr.assign(1, 0);
+    h.fst_part.clear();
+    h.fst.clear();
     h.lops.clear();
     h.lred_ptr.assign(1, 0);
     h.lred.clear();
@@ -630,16 +646,27 @@ static void build_factor_jobs(HostMech &h) {
         std::vector<int> idx(jobs.size());
         for (size_t j = 0; j < jobs.size(); j++) idx[j] = (int)j;
         balance_level(idx, 0, (int)idx.size(), NL, [&](int j) { return (int)jobs[j].ops.size() + 2; });
-        for (int j : idx) {
-            const Job &jb = jobs[j];
-            if (jb.ops.size() > 0xffff) throw std::runtime_error("factor job too long");
-            h.ljob.push_back((int)h.lops.size());
-            h.ljob.push_back((int)jb.ops.size() | (jb.ns << 16));
-            h.ljob.push_back(jb.row | (jb.recip << 16));
-            h.ljob.push_back(jb.pbase);
-            h.lops.insert(h.lops.end(), jb.ops.begin(), jb.ops.end());
+        // the jobs of lane l are idx[l], idx[l + NL], ...: one op list per lane
+        std::vector<std::vector<uint32_t>> lists(NL);
+        for (size_t j = 0; j < idx.size(); j++) {
+            const Job &jb = jobs[idx[j]];
+            std::vector<uint32_t> &v = lists[j % NL];
+            for (uint32_t op : jb.ops) {
+                if (!(op & CAMP_OP_DIV) && (op & 0x8000u)) {  // its slot among the level's partials
+                    const int slot = jb.pbase + (int)(op & 0x7fffu);
+                    if (slot > 0x7fff) throw std::runtime_error("factor partials do not fit their field");
+                    op = (op & 0xFFFF8000u) | (uint32_t)slot;
+                }
+                v.push_back(op);
+            }
+            if (jb.recip) v.push_back(((uint32_t)CAMP_OP_NOSRC << 16) | (uint32_t)h.udiag[jb.row]);
         }
-        h.ljob_ptr.push_back((int)h.ljob.size() / 4);
+        size_t steps = 0;
+        for (auto &v : lists) steps = std::max(steps, v.size());
+        for (size_t q = 0; q < steps; q++)
+            for (auto &v : lists) h.fst.push_back(q < v.size() ? v[q] : kFactorNop);
+        h.fst_ptr.push_back((int)(h.fst.size() / NL));
+        h.fst_part.push_back(lpart);
         // the level's tails, stored after its jobs
         for (size_t k = h.lred_ptr.back(); k < h.lred.size() / 4; k++) {
             const int i = h.ltail_rows[k];
@@ -648,6 +675,37 @@ static void build_factor_jobs(HostMech &h) {
             h.lops.insert(h.lops.end(), h.fops.begin() + h.fops_ptr[i] + from, h.fops.begin() + h.fops_ptr[i + 1]);
         }
         h.lred_ptr.push_back((int)h.lred.size() / 4);
+    }
+    h.fst.insert(h.fst.end(), NL, kFactorNop);
+}
+
+// One level's substitution rows as passes over the lanes (DevMech::sub_pass):
+// jobs (first entry, count, destination row) in order, NL a pass; end(j) is
+// the row word of job j.
+struct SubstJob { int first, count, dst; };
+template <class End>
+static void subst_passes(HostMech &h, const std::vector<SubstJob> &jobs, const std::vector<int> &off,
+                         const std::vector<int> &col, bool split, End end) {
+    const size_t NL = h.lanes;
+    for (size_t b = 0; b < jobs.size(); b += NL) {
+        int steps = 0;
+        for (size_t j = b; j < std::min(jobs.size(), b + NL); j++) steps = std::max(steps, (jobs[j].count + 1) / 2);
+        const size_t first = h.sub.size() / 2 / NL;
+        if (steps > 0xfff || first > 0x1ffff) throw std::runtime_error("substitution passes do not fit their fields");
+        const bool last = b + NL >= jobs.size();
+        auto entry = [&](size_t l, int q) {
+            if (b + l >= jobs.size() || q >= jobs[b + l].count) return -1;
+            return field16(off[jobs[b + l].first + q]) | (field16(col[jobs[b + l].first + q]) << 16);
+        };
+        for (size_t l = 0; l < NL; l++) {
+            h.sub_pass.push_back(b + l < jobs.size() ? end(jobs[b + l]) : -1);
+            h.sub_pass.push_back(entry(l, 0));
+            h.sub_pass.push_back(entry(l, 1));
+            h.sub_pass.push_back(steps | (last ? 0x1000 : 0) | (last && split ? 0x2000 : 0) | (int)(first << 14));
+        }
+        for (int t = 1; t < steps; t++)
+            for (size_t l = 0; l < NL; l++)
+                for (int e = 0; e < 2; e++) h.sub.push_back(entry(l, 2 * t + e));
     }
 }
 
@@ -722,14 +780,28 @@ static void build_tables(HostMech &h) {
         std::vector<int> order(jobs.size());
         for (size_t j = 0; j < jobs.size(); j++) order[j] = (int)j;
         std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return jobs[a].count > jobs[b].count; });
-        std::vector<std::vector<int>> lanes(NL);
-        std::vector<long long> load(NL, 0);
+        // entry pairs per job, heaviest first into the first lane with room,
+        // at the smallest room for which that fits
+        auto pairs = [&](int j) { return std::max(1, (jobs[j].count + 1) / 2); };
+        long long sum = 0;
+        int longest = 1;
         for (int j : order) {
-            int best = 0;
-            for (int l = 1; l < NL; l++)
-                if (load[l] < load[best]) best = l;
-            lanes[best].push_back(j);
-            load[best] += jobs[j].count + 2;  // entries plus the per-sum cost
+            sum += pairs(j);
+            longest = std::max(longest, pairs(j));
+        }
+        std::vector<std::vector<int>> lanes;
+        for (long long room = std::max<long long>(longest, (sum + NL - 1) / NL);; room++) {
+            lanes.assign(NL, {});
+            std::vector<long long> load(NL, 0);
+            bool fits = true;
+            for (int j : order) {
+                int l = 0;
+                while (l < NL && load[l] + pairs(j) > room) l++;
+                if (l == NL) { fits = false; break; }
+                lanes[l].push_back(j);
+                load[l] += pairs(j);
+            }
+            if (fits) break;
         }
         h.flane_ptr.assign(1, 0);
         h.flane_pos.clear();
@@ -755,8 +827,32 @@ static void build_tables(HostMech &h) {
         if ((double)cnt >= 0.75 * (double)(n - d) * (double)(n - d)) { h.d = d; break; }
     }
     if (n - h.d > 128) h.d = n - 128;  // the substitution keeps at most 4 block rows per lane
+    // The block's rows are padded to a stride of 4 mod 8 values (16-byte row
+    // pieces without bank conflicts).  Where that padding would take a
+    // mechanism over a limit that compact rows respect, the block shrinks
+    // until it does not.
+    auto stride = [](int D) { return D > 0 ? ((D + 3) & ~7) + 4 : 0; };
+    auto stored = [&](int d, int LD) {  // LU values stored with the block starting at d
+        int sp = 0;
+        for (int i = 0; i < n; i++)
+            for (int q = h.lu_rowptr[i]; q < h.lu_rowptr[i + 1]; q++) sp += (i < d || h.lu_colidx[q] < d);
+        return ((sp + 3) & ~3) + (n - d) * LD;
+    };
+    {
+        const int compact = stored(h.d, (n - h.d) | 1);
+        // partials and the water parameter's values at most, besides the LU
+        const int scratch = 3 * 2048 + 4 * n;
+        auto bytes = [&](int nlu, int elem) { return cell_smem(n, R, h.n_rev, nlu, elem, scratch, 1 << 20, 0, 0, h.lanes).bytes; };
+        auto fits = [&](int d) {
+            const int s = stored(d, stride(n - d));
+            if (s <= compact) return true;
+            return s <= 32767 && bytes(s, 4) <= CAMP_MAX_SMEM &&
+                   (bytes(s, 8) <= CAMP_MAX_SMEM || cell_smem(n, R, h.n_rev, compact, 8, 0, 1 << 20, 0, 0, h.lanes).bytes > CAMP_MAX_SMEM);
+        };
+        while (h.d < n && !fits(h.d)) h.d++;
+    }
     h.D = n - h.d;
-    h.LD = h.D % 2 ? h.D : h.D + 1;
+    h.LD = stride(h.D);
 
     // storage offsets: sparse rows < d, the L21 part of rows >= d, then the block
     std::vector<int> lu_off(h.lu_colidx.size(), -1);
@@ -990,12 +1086,12 @@ static void build_tables(HostMech &h) {
     // products a second pass subtracts in a fixed order.
     {
         const int NL = h.lanes;
-        h.slev_ptr.assign(1, 0);
-        h.sjob.clear();
+        h.sub_pass.clear();
+        h.sub.clear();
         h.ssplit_ptr.assign(1, 0);
         h.ssplit.clear();
         h.n_spart = 0;
-        struct Job { int first, count, dst; };
+        using Job = SubstJob;
         for (size_t l = 0; l + 1 < h.flev_ptr.size(); l++) {
             std::vector<int> rows;
             long long total = 0;
@@ -1026,12 +1122,14 @@ static void build_tables(HostMech &h) {
             std::vector<int> idx(jobs.size());
             for (size_t j = 0; j < jobs.size(); j++) idx[j] = (int)j;
             balance_level(idx, 0, (int)idx.size(), NL, [&](int j) { return jobs[j].count + 1; });
+            std::vector<Job> sorted;
             for (int j : idx) {
                 if (jobs[j].dst > 0xffff || jobs[j].count > 0xffff) throw std::runtime_error("substitution jobs do not fit 16-bit fields");
-                h.sjob.push_back(jobs[j].first);
-                h.sjob.push_back(jobs[j].dst | (jobs[j].count << 16));
+                sorted.push_back(jobs[j]);
             }
-            h.slev_ptr.push_back((int)h.sjob.size() / 2);
+            // passes of similar rows: longest first
+            std::stable_sort(sorted.begin(), sorted.end(), [](const Job &a, const Job &b) { return a.count > b.count; });
+            subst_passes(h, sorted, h.sl_off, h.sl_col, np > 0, [](const Job &j) { return j.dst; });
             h.ssplit_ptr.push_back((int)h.ssplit.size() / 2);
         }
     }
@@ -1046,14 +1144,19 @@ static void build_tables(HostMech &h) {
         bl[i] = lv + 1;
         maxb = std::max(maxb, bl[i]);
     }
-    h.blev_ptr.assign(1, 0);
-    h.brow.clear();
+    h.n_fpass = (int)(h.sub_pass.size() / 4 / h.lanes);
     for (int l = 0; l <= maxb; l++) {
-        for (int i = 0; i < h.d; i++) if (bl[i] == l) h.brow.push_back(i);
-        h.blev_ptr.push_back((int)h.brow.size());
-        const int b = h.blev_ptr[h.blev_ptr.size() - 2], e = h.blev_ptr.back();
-        balance_level(h.brow, b, e, h.lanes, [&](int i) { return h.su_ptr[i + 1] - h.su_ptr[i] + 1; });
+        std::vector<int> rows;
+        for (int i = 0; i < h.d; i++) if (bl[i] == l) rows.push_back(i);
+        std::vector<SubstJob> jobs;
+        for (int i : rows) jobs.push_back({h.su_ptr[i], h.su_ptr[i + 1] - h.su_ptr[i], i});
+        std::stable_sort(jobs.begin(), jobs.end(), [](const SubstJob &a, const SubstJob &b) { return a.count > b.count; });
+        subst_passes(h, jobs, h.su_off, h.su_col, false,
+                     [&](const SubstJob &j) { return j.dst | (h.udiag[j.dst] << 16); });
     }
+    h.n_bpass = (int)(h.sub_pass.size() / 4 / h.lanes) - h.n_fpass;
+    h.sub.insert(h.sub.end(), 2 * (size_t)h.lanes, -1);
+    h.sub_pass.insert(h.sub_pass.end(), 4 * (size_t)h.lanes, -1);
 }
 
 // Bounds of every index the device tables hold, checked once per mechanism
@@ -1092,8 +1195,6 @@ static void validate_tables(const HostMech &h) {
     }
     // forcing gather
     const int nf = (int)h.fk.size();
-    for (int q = 0; q < nf; q++)
-        if (!in(f16(h.fpk[q]), 0, R) || !in(h16(h.fpk[q]), 0, (int)h.fcoef.size())) fail("fpk");
     const int nj = (int)h.fjob.size() / 2;
     if (h.flane_ptr.front() != 0 || h.flane_ptr.back() != nj) fail("flane_ptr");
     for (size_t l = 0; l + 1 < h.flane_ptr.size(); l++) if (h.flane_ptr[l] > h.flane_ptr[l + 1]) fail("flane_ptr order");
@@ -1101,36 +1202,57 @@ static void validate_tables(const HostMech &h) {
         const int first = h.fjob[2 * i], dst = f16(h.fjob[2 * i + 1]), cnt = h16(h.fjob[2 * i + 1]);
         if (!in(first, 0, nf + 1) || first + cnt > nf || !in(dst, 0, n + h.n_fpart)) fail("fjob");
     }
+    if (h.gth.size() != (size_t)(h.n_gstep + 2) * h.lanes * 2 || h.gcf.size() != h.gth.size()) fail("gth size");
+    for (size_t q = 0; q < h.gth.size(); q += 2) {
+        for (int e = 0; e < 2; e++) {
+            const int w = (h.gth[q] >> (16 * e)) & 0xffff;
+            if (w & 0x8000 ? w != 0x8000 : !in(w, 0, R)) fail("gth");
+        }
+        if (!in(h.gth[q + 1], -1, n + h.n_fpart)) fail("gth destination");
+    }
     for (size_t i = 0; i < h.fsplit.size() / 2; i++) {
         const int pos = h.fsplit[2 * i], first = f16(h.fsplit[2 * i + 1]), cnt = h16(h.fsplit[2 * i + 1]);
         if (!in(pos, 0, n) || first + cnt > h.n_fpart) fail("fsplit");
     }
     // Jacobian lists
     const int nnzJ = (int)h.colidx.size();
-    for (size_t i = 0; i < h.jl_rec.size() / 4; i++) {
-        const int *r = &h.jl_rec[4 * i];
+    for (int w = 0; 32 * w < h.lanes; w++)
+        if ((size_t)h.n_jstep[w] * h.lanes * 4 > h.jls.size() || h.jlc.size() * 4 != h.jls.size()) fail("jls size");
+    for (int l = 0; l < h.lanes; l++) {  // every list ends within the stored steps
+        size_t i = l;
+        while (i < h.jlc.size() && !(h.jls[4 * i + 2] & (1 << 18))) i += h.lanes;
+        if (i >= h.jlc.size() || (int)(i / h.lanes) >= h.n_jstep[l / 32]) fail("jls end");
+    }
+    for (size_t i = 0; i < h.jls.size() / 4; i++) {
+        const int *r = &h.jls[4 * i];
         const int k = (int)(short)(r[1] & 0xffff), o1 = h16(r[1]), o2 = f16(r[3]), t = h16(r[3]);
-        if (!in(k, -h.n_rev, R) || (o1 != NONE && !in(o1, 0, n)) || (o2 != NONE && !in(o2, 0, n))) fail("jl_rec");
-        if (!in(r[2] & 0xffff, 0, nlu) || !in(t, 0, nnzJ)) fail("jl_rec target");
+        if (!in(k, -h.n_rev, R) || (o1 != NONE && !in(o1, 0, n)) || (o2 != NONE && !in(o2, 0, n))) fail("jls");
+        if (!in(r[2] & 0xffff, 0, nlu) || !in(t, 0, nnzJ)) fail("jls target");
     }
     // LU: storage layout, factorisation jobs, substitution lists
-    if (h.dbase + h.D * h.LD > nlu || h.d + h.D != n) fail("dense block");
+    if (h.dbase + h.D * h.LD > nlu || h.d + h.D != n || h.D > 128) fail("dense block");
+    if (h.D > 0 && (h.LD < h.D || h.LD % 8 != 4 || h.dbase % 4 != 0)) fail("dense block alignment");
     for (int i = 0; i < h.d; i++) if (!in(h.udiag[i], 0, nlu)) fail("udiag");
     const int nops = (int)h.lops.size();
-    for (size_t j = 0; j < h.ljob.size() / 4; j++) {
-        const int *jb = &h.ljob[4 * j];
-        const int cnt = f16(jb[1]), ns = h16(jb[1]), row = f16(jb[2]);
-        if (jb[0] < 0 || jb[0] + cnt > nops || !in(row, 0, n) || (ns > 0 && jb[3] + ns > h.n_lpart))
-            fail("ljob");
-        for (int q = jb[0]; q < jb[0] + cnt; q++) {
-            const uint32_t op = h.lops[q];
-            const int t = (int)(op & 0xffffu), src = (int)((op >> 16) & 0x7fffu);
-            if (!in(src, 0, nlu)) fail("lops source");
+    if (h.fst.size() != ((size_t)h.fst_ptr.back() + 1) * h.lanes || h.fst_part.size() + 1 != h.fst_ptr.size()) fail("fst size");
+    for (size_t L = 0; L + 1 < h.fst_ptr.size(); L++) {
+        if (h.fst_ptr[L] > h.fst_ptr[L + 1] || !in(h.fst_part[L], 0, h.n_lpart + 1)) fail("fst_ptr");
+        for (size_t q = (size_t)h.fst_ptr[L] * h.lanes; q < (size_t)h.fst_ptr[L + 1] * h.lanes; q++) {
+            const uint32_t op = h.fst[q];
+            const int t = (int)(op & 0xffffu), src = CAMP_OP_SRC(op);
+            if (src == CAMP_OP_NOSRC) {
+                if (op != kFactorNop && ((op & CAMP_OP_DIV) || !in(t, 0, nlu))) fail("fst pivot");
+                continue;
+            }
+            if (!in(src, 0, nlu)) fail("fst source");
             if ((t & 0x8000) && !(op & CAMP_OP_DIV)) {
-                if (!in(jb[3] + (t & 0x7fff), 0, h.n_lpart) || (t & 0x7fff) >= ns) fail("lops partial");
-            } else if (!in(t, 0, nlu)) fail("lops target");
+                if (h.lanes <= 32 || !in(t & 0x7fff, 0, h.fst_part[L])) fail("fst partial");
+            } else if (!in(t, 0, nlu)) fail("fst target");
         }
     }
+    for (size_t q = (size_t)h.fst_ptr.back() * h.lanes; q < h.fst.size(); q++) if (h.fst[q] != kFactorNop) fail("fst padding");
+    for (uint32_t op : h.lops)
+        if (!in(CAMP_OP_SRC(op), 0, nlu) || !in((int)(op & 0xffffu), 0, nlu)) fail("lops");
     for (size_t k = 0; k < h.lred.size() / 4; k++) {
         const int *rd = &h.lred[4 * k];
         const int ns = f16(rd[2]), nch = h16(rd[2]);
@@ -1140,19 +1262,31 @@ static void validate_tables(const HostMech &h) {
         for (int q = h.ltail[2 * k]; q < h.ltail[2 * k] + h.ltail[2 * k + 1]; q++)
             if ((h.lops[q] & 0x8000u) && !(h.lops[q] & CAMP_OP_DIV)) fail("tail op with a partial target");
     }
-    auto check_pack = [&](const std::vector<int> &pk, const char *what) {
-        for (int w : pk) if (!in(f16(w), 0, nlu) || !in(h16(w), 0, n)) fail(what);
-    };
-    check_pack(h.sl_pack, "sl_pack");
-    check_pack(h.su_pack, "su_pack");
-    const int nsl = (int)h.sl_pack.size();
-    for (size_t r = 0; r < h.sjob.size() / 2; r++) {
-        const int first = h.sjob[2 * r], dst = f16(h.sjob[2 * r + 1]), cnt = h16(h.sjob[2 * r + 1]);
-        if (first < 0 || first + cnt > nsl || !in(dst, 0, n + h.n_spart)) fail("sjob");
+    const int n_pass = h.n_fpass + h.n_bpass, n_sub = (int)(h.sub.size() / 2 / h.lanes);
+    if (h.sub_pass.size() != (size_t)(n_pass + 1) * h.lanes * 4 || h.sub.size() % (2 * (size_t)h.lanes)) fail("sub size");
+    int split_levels = 0, levels = 0;
+    for (int p = 0; p < n_pass; p++) {
+        const bool back = p >= h.n_fpass;
+        const int *r0 = &h.sub_pass[(size_t)p * h.lanes * 4];
+        const int steps = r0[3] & 0xfff, first = (int)((unsigned)r0[3] >> 14);
+        if (first + std::max(steps, 1) > n_sub) fail("sub_pass");
+        if (!back && (r0[3] & 0x1000)) { levels++; split_levels += (r0[3] & 0x2000) != 0; }
+        for (int l = 0; l < h.lanes; l++) {
+            const int *r = r0 + 4 * l;
+            if (r[3] != r0[3] || r[0] < -1) fail("sub_pass");
+            if (r[0] >= 0 && (!in(f16(r[0]), 0, back || h.lanes <= 32 ? n : n + h.n_spart) ||
+                              !in(h16(r[0]), 0, back ? nlu : 1)))
+                fail("sub_pass row");
+            for (int e = 1; e < 3; e++)
+                if (r[e] < -1 || (r[e] >= 0 && (!in(f16(r[e]), 0, nlu) || !in(h16(r[e]), 0, n)))) fail("sub_pass entry");
+        }
     }
+    if (levels + 1 != (int)h.ssplit_ptr.size() || (split_levels > 0) != (h.ssplit.size() > 0)) fail("sub levels");
+    if (n_pass > 0 && n_pass != h.n_fpass && !(h.sub_pass[(size_t)(n_pass - 1) * h.lanes * 4 + 3] & 0x1000)) fail("sub levels");
+    for (int w : h.sub)
+        if (w < -1 || (w >= 0 && (!in(f16(w), 0, nlu) || !in(h16(w), 0, n)))) fail("sub");
     for (size_t k = 0; k < h.ssplit.size() / 2; k++)
         if (!in(h.ssplit[2 * k], 0, n) || f16(h.ssplit[2 * k + 1]) + h16(h.ssplit[2 * k + 1]) > h.n_spart) fail("ssplit");
-    for (int i : h.brow) if (!in(i, 0, h.d)) fail("brow");
     // water parameter
     if (!h.el_phase.empty()) {
         const int S = h.n_sections, n_el = (int)h.el_phase.size(), n_pp = (int)h.pp.size() / 4;
@@ -1337,48 +1471,41 @@ std::vector<unsigned char> pack_tables(const HostMech &h, DevMech &dm, const uns
     dm.rnp = pk.put(h.rnp);
     dm.n_rev = h.n_rev;
     dm.rrev = pk.put(h.rrev);
-    dm.flane_ptr = pk.put(h.flane_ptr);
     dm.nnzJ = (int)h.colidx.size();
-    dm.jk = pk.put(h.jk);
-    dm.jo = pk.put(h.jo);
-    dm.jc = pk.put(h.jc);
     dm.nlu = h.nlu;
     dm.d = h.d;
     dm.D = h.D;
     dm.LD = h.LD;
     dm.dbase = h.dbase;
     dm.n_flev = (int)h.flev_ptr.size() - 1;
-    dm.ljob_ptr = pk.put(h.ljob_ptr);
-    dm.ljob = reinterpret_cast<const int4 *>(pk.put(h.ljob));
+    dm.fst_ptr = pk.put(h.fst_ptr);
+    dm.fst_part = pk.put(h.fst_part);
+    dm.fst = pk.put(h.fst);
     dm.lops = pk.put(h.lops);
     dm.lred_ptr = pk.put(h.lred_ptr);
     dm.lred = reinterpret_cast<const int4 *>(pk.put(h.lred));
     dm.lred_off = pk.put(h.lred_off);
     dm.ltail = reinterpret_cast<const int2 *>(pk.put(h.ltail));
-    dm.n_slev = (int)h.slev_ptr.size() - 1;
-    dm.slev_ptr = pk.put(h.slev_ptr);
-    dm.sjob = reinterpret_cast<const int2 *>(pk.put(h.sjob));
+    dm.sub_pass = reinterpret_cast<const int4 *>(pk.put(h.sub_pass));
+    dm.sub = reinterpret_cast<const int2 *>(pk.put(h.sub));
+    dm.n_fpass = h.n_fpass;
+    dm.n_bpass = h.n_bpass;
     dm.ssplit_ptr = pk.put(h.ssplit_ptr);
     dm.ssplit = reinterpret_cast<const int2 *>(pk.put(h.ssplit));
     // partials in doubles: the factor's are LU-precision values, at most 8 bytes
     dm.n_part = std::max(std::max(h.n_fpart, h.n_spart), h.n_lpart);
-    dm.n_blev = (int)h.blev_ptr.size() - 1;
-    dm.blev_ptr = pk.put(h.blev_ptr);
-    dm.brow = pk.put(h.brow);
-    dm.su_ptr = pk.put(h.su_ptr);
     dm.udiag = pk.put(h.udiag);
     dm.perm = pk.put(h.perm);
     dm.rpack = reinterpret_cast<const int4 *>(pk.put(h.rpack));
-    dm.fpk = pk.put(h.fpk);
-    dm.fcoef = pk.put(h.fcoef);
-    dm.fjob = reinterpret_cast<const int2 *>(pk.put(h.fjob));
+    dm.gth = reinterpret_cast<const int2 *>(pk.put(h.gth));
+    dm.gcf = reinterpret_cast<const double2 *>(pk.put(h.gcf));
+    dm.n_gstep = h.n_gstep;
+    dm.n_fpart = h.n_fpart;
     dm.n_fsplit = (int)h.fsplit.size() / 2;
     dm.fsplit = reinterpret_cast<const int2 *>(pk.put(h.fsplit));
-    dm.jnz = reinterpret_cast<const int4 *>(pk.put(h.jnz));
-    dm.sl_pack = pk.put(h.sl_pack);
-    dm.jl_ptr = pk.put(h.jl_ptr);
-    dm.jl_rec = reinterpret_cast<const int4 *>(pk.put(h.jl_rec));
-    dm.su_pack = pk.put(h.su_pack);
+    dm.jls = reinterpret_cast<const int4 *>(pk.put(h.jls));
+    dm.jlc = pk.put(h.jlc);
+    std::copy(h.n_jstep, h.n_jstep + 8, dm.n_jstep);
     dm.n_wsec = h.el_phase.empty() ? 0 : h.n_sections;
     dm.n_el = (int)h.el_phase.size();
     dm.rh_slot = h.rh_slot;
@@ -1396,6 +1523,9 @@ std::vector<unsigned char> pack_tables(const HostMech &h, DevMech &dm, const uns
     dm.ch = reinterpret_cast<const int4 *>(pk.put(h.ch));
     dm.n_pw = h.n_pw;
     dm.n_pw64 = h.n_pw64;
+    for (int elem : {4, 8})
+        (elem == 4 ? dm.smem4 : dm.smem8) =
+            cell_smem(dm.n, dm.R, dm.n_rev, dm.nlu, elem, dm.n_part, dm.n_fpart, dm.n_pw, dm.n_pw64, dm.lanes);
     bdf_coefficients(dm);
     return pk.img;
 }

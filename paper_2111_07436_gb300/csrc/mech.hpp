@@ -50,26 +50,31 @@ struct HostMech {
     std::vector<int> fptr, fk;
     std::vector<double> fc;
     std::vector<int> flane_ptr, flane_pos;
-    std::vector<int> rpack, jnz, sl_pack, su_pack;  // int4 records as 4 ints
-    std::vector<int> fpk, fjob;   // forcing gather entries and lane jobs (see DevMech)
+    std::vector<int> rpack;       // int4 records as 4 ints
+    std::vector<int> fjob;        // forcing sums as lane jobs: first entry, position | entry count << 16
+    std::vector<int> gth;         // the same as one flat list per lane (see DevMech)
+    int n_gstep = 0;
     std::vector<int> fsplit;      // split sums, 2 ints each (see DevMech)
     int n_fpart = 0;
-    std::vector<double> fcoef;
-    std::vector<int> jl_ptr, jl_rec;
+    std::vector<double> gcf;
+    std::vector<int> jls;         // Jacobian entry lists (see DevMech)
+    std::vector<double> jlc;
+    int n_jstep[8] = {};
     std::vector<int> jptr, jdst, jdiag, jk, jo;
     std::vector<double> jc;
     int nlu = 0, d = 0, D = 0, LD = 0, dbase = 0;
     std::vector<int> flev_ptr, frow, fops_ptr;
     std::vector<uint32_t> fops;
-    // the factorisation as lane jobs (see DevMech)
-    std::vector<int> ljob_ptr, ljob, lred_ptr, lred, lred_off, ltail, ltail_rows;
-    std::vector<uint32_t> lops;
+    // the factorisation as lane lists (see DevMech)
+    std::vector<int> fst_ptr, fst_part, lred_ptr, lred, lred_off, ltail, ltail_rows;
+    std::vector<uint32_t> fst, lops;
     int n_lpart = 0;
     std::vector<int> sl_ptr, sl_off, sl_col;
-    // forward substitution: lane jobs by level, split rows (see DevMech)
-    std::vector<int> slev_ptr, sjob, ssplit_ptr, ssplit;
+    // substitution: passes over the lanes by level, split rows (see DevMech)
+    std::vector<int> sub_pass, sub, ssplit_ptr, ssplit;
+    int n_fpass = 0, n_bpass = 0;
     int n_spart = 0;
-    std::vector<int> blev_ptr, brow, su_ptr, su_off, su_col, udiag;
+    std::vector<int> su_ptr, su_off, su_col, udiag;
     long long factor_updates = 0;  // multiply-adds one device factorisation executes
     // algorithmic work of the method, from the symbolic structure
     long long flops_forcing = 0;   // one f(y): rate products + stoichiometric sums
