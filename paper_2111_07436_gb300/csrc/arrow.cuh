@@ -176,7 +176,7 @@ __device__ inline void arrow_particle_assemble(const ArrowDev &a, int p, const d
     for (int k = 0; k < a.Rp; k++) {
         const int4 r0 = __ldg(a.prec + 3 * k), r1 = __ldg(a.prec + 3 * k + 1), r2 = __ldg(a.prec + 3 * k + 2);
         const int fac[6] = {r1.x, r1.y, r1.z, r2.x, r2.y, r2.z};
-        const LT kf = (LT)kfp[(size_t)k * P + p], kr = (LT)krp[(size_t)k * P + p];
+        const LT kf = to_lu<LT>(kfp[(size_t)k * P + p]), kr = to_lu<LT>(krp[(size_t)k * P + p]);
         LT d[6];
 #pragma unroll
         for (int q = 0; q < 6; q++) {
@@ -263,7 +263,7 @@ __device__ inline void arrow_particle_forward(const ArrowDev &a, int p, const LT
     for (int c = 0; c < nc; c++) {
         LT s = (LT)0;
         for (int j = 0; j < np; j++) s += LGp[((size_t)c * np + j) * P + p] * y[j];
-        fw[c] += (double)s;
+        fw[c] += from_lu(s);
     }
 }
 
@@ -316,12 +316,12 @@ __device__ int arrow_integrate_cell(const DevMech &mt, const ArrowDev &a, ArrowS
     double zg[QMAX + 1], eg = 0.0, epg = 0.0, wg = 0.0, fg = 0.0;
 
     // inputs must be finite
-    double nbad = 0.0;
-    for (int i = lane; i < a.n_env; i += L) nbad += !finite_bits(env[i]);
+    int bad_in = 0;  // counted in integers: an FP64 add is a warp's for 64 cycles
+    for (int i = lane; i < a.n_env; i += L) bad_in += !finite_bits(env[i]);
     for (int p = lane; p < a.P; p += L)
         for (int i = 0; i < np; i++) {
             const double v = y_cell[species(i, p)];
-            nbad += !finite_bits(v);
+            bad_in += !finite_bits(v);
             Z(0, i, p) = v;
             for (int j = 1; j <= QMAX; j++) Z(j, i, p) = 0.0;
             E(i, p) = EP(i, p) = 0.0;
@@ -330,13 +330,13 @@ __device__ int arrow_integrate_cell(const DevMech &mt, const ArrowDev &a, ArrowS
     for (int j = 0; j <= QMAX; j++) zg[j] = 0.0;
     if (gas_own) {
         zg[0] = y_cell[tid];
-        nbad += !finite_bits(zg[0]);
+        bad_in += !finite_bits(zg[0]);
     }
     auto fail_early = [&](int code) {
         if (step_io && lane == 0) *step_io = 0.0;
         return code;
     };
-    if (cluster_sum1(sm, cl, nbad, par) != 0.0) return fail_early(ST_NONFINITE);
+    if (cluster_sum1(sm, cl, (double)bad_in, par) != 0.0) return fail_early(ST_NONFINITE);
 
     // rate constants: the particles' (own), the gas processes' (gas warp)
     for (int p = lane; p < a.P; p += L) {
@@ -396,17 +396,19 @@ __device__ int arrow_integrate_cell(const DevMech &mt, const ArrowDev &a, ArrowS
         double part[CAMP_ARROW_MAX_C + 1];
         for (int q = 0; q <= nc; q++) part[q] = 0.0;
         double yl[ARROW_MAX_LOC], fl[ARROW_MAX_LOC];
+        int bad_f = 0;
         for (int p = lane; p < a.P; p += L) {
             for (int i = 0; i < np; i++) yl[i] = Z(0, i, p) + b * F(i, p);
             for (int q = 0; q < nc; q++) yl[np + q] = sm.ygas[__ldg(a.coupled + q)];
             arrow_particle_forcing(a, p, c.kfp, c.krp, yl, fl);
             for (int i = 0; i < np; i++) {
-                part[nc] += !finite_bits(fl[i]);
+                bad_f += !finite_bits(fl[i]);
                 if (diff) EP(i, p) = fl[i] - F(i, p);
                 else F(i, p) = fl[i];
             }
             for (int q = 0; q < nc; q++) part[q] += fl[np + q];
         }
+        part[nc] = (double)bad_f;
         gas_rates();
         double red[CAMP_ARROW_MAX_C + 1];
         cluster_sum(sm, cl, part, nc + 1, par, red);
@@ -532,12 +534,12 @@ __device__ int arrow_integrate_cell(const DevMech &mt, const ArrowDev &a, ArrowS
         LT gg[CAMP_ARROW_MAX_C * CAMP_ARROW_MAX_C];
         LT yl[ARROW_MAX_LOC];
         for (int p = lane; p < a.P; p += L) {
-            for (int i = 0; i < np; i++) yl[i] = (LT)Z(0, i, p);
-            for (int k = 0; k < nc; k++) yl[np + k] = (LT)sm.ygas[__ldg(a.coupled + k)];
+            for (int i = 0; i < np; i++) yl[i] = to_lu<LT>(Z(0, i, p));
+            for (int k = 0; k < nc; k++) yl[np + k] = to_lu<LT>(sm.ygas[__ldg(a.coupled + k)]);
             for (int v = 0; v < nc * nc; v++) gg[v] = (LT)0;
             arrow_particle_assemble<LT>(a, p, c.kfp, c.krp, yl, g, c.lu, gg);
             const bool bad = arrow_particle_factor<LT>(a, p, c.lu, gg);
-            for (int v = 0; v < nc * nc; v++) part[v] += (double)gg[v];
+            for (int v = 0; v < nc * nc; v++) part[v] += from_lu(gg[v]);
             part[nc * nc] += bad ? 1.0 : 0.0;
         }
         double red[ARROW_RED];
@@ -638,17 +640,22 @@ __device__ int arrow_integrate_cell(const DevMech &mt, const ArrowDev &a, ArrowS
                     double part[2 * CAMP_ARROW_MAX_C + 1];
                     for (int v = 0; v <= 2 * nc; v++) part[v] = 0.0;
                     double yl[ARROW_MAX_LOC], fl[ARROW_MAX_LOC];
+                    int bad_f = 0;
                     for (int p = lane; p < a.P; p += L) {
-                        for (int i = 0; i < np; i++) yl[i] = Z(0, i, p) + (it ? E(i, p) : 0.0);
+                        for (int i = 0; i < np; i++) yl[i] = Z(0, i, p);
+                        if (it)
+                            for (int i = 0; i < np; i++) yl[i] += E(i, p);
                         for (int k = 0; k < nc; k++) yl[np + k] = sm.ygas[__ldg(a.coupled + k)];
                         arrow_particle_forcing(a, p, c.kfp, c.krp, yl, fl);
                         for (int i = 0; i < np; i++) {
-                            part[2 * nc] += !finite_bits(fl[i]);
-                            X(i, p) = to_lu<LT>(-((it ? E(i, p) : 0.0) - gamma * fl[i] + Z(1, i, p) * rl1));
+                            bad_f += !finite_bits(fl[i]);
+                            const double r = fma(-gamma, fl[i], it ? E(i, p) : 0.0);
+                            X(i, p) = to_lu<LT>(-fma(Z(1, i, p), rl1, r));
                         }
                         for (int k = 0; k < nc; k++) part[k] += fl[np + k];
                         arrow_particle_forward<LT>(a, p, c.lu, c.xp, part + nc);
                     }
+                    part[2 * nc] = (double)bad_f;
                     gas_rates();
                     double red[2 * CAMP_ARROW_MAX_C + 1];
                     cluster_sum(sm, cl, part, 2 * nc + 1, par, red);
@@ -686,14 +693,17 @@ __device__ int arrow_integrate_cell(const DevMech &mt, const ArrowDev &a, ArrowS
                     // and the weighted sum of squares of e (the error test's,
                     // in the same order as a pass of its own would take)
                     double s2[3] = {0.0, red[2 * nc] + gnf, 0.0};
+                    int bad_x = 0;
                     for (int p = lane; p < a.P; p += L) {
                         arrow_particle_backward<LT>(a, p, c.lu, c.xp, sm.xgas);
                         for (int i = 0; i < np; i++) {
                             LT xl = X(i, p) * scale;
-                            const double en = (it ? E(i, p) : 0.0) + from_lu(xl), wv = Wt(i, p);
+                            double en = from_lu(xl);
+                            const double wv = Wt(i, p);
+                            if (it) en += E(i, p);
                             E(i, p) = en;
-                            s2[0] += (double)upd_term(xl, wv);
-                            s2[1] += !isfinite(xl);
+                            s2[0] += from_lu(upd_term(xl, norm_weight<LT>(wv)));
+                            bad_x += !isfinite(xl);
                             const double v = en * wv;
                             s2[2] += v * v;
                         }
@@ -701,10 +711,11 @@ __device__ int arrow_integrate_cell(const DevMech &mt, const ArrowDev &a, ArrowS
                     if (gas_own) {
                         LT xl = sm.xgas[tid] * scale;
                         eg += from_lu(xl);
-                        s2[0] += (double)upd_term(xl, wg);
-                        s2[1] += !isfinite(xl);
+                        s2[0] += from_lu(upd_term(xl, norm_weight<LT>(wg)));
+                        bad_x += !isfinite(xl);
                         s2[2] += (eg * wg) * (eg * wg);
                     }
+                    s2[1] += (double)bad_x;
                     double r2[3];
                     cluster_sum(sm, cl, s2, 3, par, r2);
                     esum = r2[2];
@@ -769,11 +780,12 @@ __device__ int arrow_integrate_cell(const DevMech &mt, const ArrowDev &a, ArrowS
         const double t_new = last ? T : t + h;
         const bool select = qwait - 1 <= 0 && t_new < T;
         double acc[3] = {0.0, 0.0, 0.0};  // non-finite count, sum (z_q w)^2, sum ((e - ep) w)^2
+        int bad_z = 0;
         for (int p = lane; p < a.P; p += L)
             for (int i = 0; i < np; i++) {
                 const double ev = E(i, p);
                 for (int j = 0; j <= q; j++) Z(j, i, p) += mt.lcoef[q][j] * ev;
-                acc[0] += !finite_bits(Z(0, i, p));
+                bad_z += !finite_bits(Z(0, i, p));
                 if (select) {
                     const double w = Wt(i, p);
                     const double zq = Z(q, i, p) * w, de = (ev - EP(i, p)) * w;
@@ -785,7 +797,7 @@ __device__ int arrow_integrate_cell(const DevMech &mt, const ArrowDev &a, ArrowS
             }
         if (gas_own) {
             for (int j = 0; j <= q; j++) zg[j] += mt.lcoef[q][j] * eg;
-            acc[0] += !finite_bits(zg[0]);
+            bad_z += !finite_bits(zg[0]);
             if (select) {
                 const double zq = zg[q] * wg, de = (eg - epg) * wg;
                 acc[1] += zq * zq;
@@ -797,6 +809,7 @@ __device__ int arrow_integrate_cell(const DevMech &mt, const ArrowDev &a, ArrowS
         t = t_new;
         nst++;
         st.ordsum += q;
+        acc[0] = (double)bad_z;
         double r3[3];
         cluster_sum(sm, cl, acc, 3, par, r3);
         if (r3[0] != 0.0) { status = ST_NONFINITE; break; }

@@ -119,8 +119,29 @@ cudaError_t camp_launch_rates(const DevMech &m, long long n_cells, const double 
     return cudaGetLastError();
 }
 
+// Whether f takes a lane a cell (k_forcing_lanes).  A warp of 32 cells takes
+// the same time however many there are, up to four warps an SM (19456
+// cells): 0.82 ms for the 72-species mechanism (186 processes), 0.056 ms for
+// 12 processes.  A warp a cell, R / 32 processes at a time, takes 0.82 ms for
+// 13000 cells of the former and 0.056 ms for 1500 of the latter (3.45 ms
+// against 5.83 ms for 65537 gas-72 cells, 0.12 against 2.2 ms of the small
+// mechanism's, before the exact powers were skipped).  One-warp cells without
+// a water parameter only: their sums are not split, so both kernels add them
+// in the same order; four warps' rates have to fit an SM.
+static bool forcing_by_lanes(const DevMech &m, long long n_cells) {
+    return m.lanes == 32 && m.n_wsec == 0 && 4 * (32 * 8 * m.R + 1024) <= 228 * 1024 &&
+           n_cells * ((m.R + 31) / 32 * 32) >= 13000LL * m.R;
+}
+
 cudaError_t camp_launch_forcing(const DevMech &m, long long n_cells, const double *state,
                                 const double *env, double *f, cudaStream_t s) {
+    if (forcing_by_lanes(m, n_cells)) {
+        const int rates = 32 * 8 * m.R;
+        cudaError_t e = cudaFuncSetAttribute(campdev::k_forcing_lanes<32>, cudaFuncAttributeMaxDynamicSharedMemorySize, rates);
+        if (e != cudaSuccess) return e;
+        campdev::k_forcing_lanes<32><<<(unsigned)((n_cells + 31) / 32), 32, rates, s>>>(m, n_cells, state, env, f);
+        return cudaGetLastError();
+    }
     if (m.n_wsec > 0) {  // the water build: 8-slot shapes only
         switch (camp_pick_shape(m.n, m.lanes) < CAMP_SHAPE_BLOCK ? 8 : camp_pick_shape(m.n, m.lanes)) {
         case 8: return forcing_npl<32, 8, true>(m, n_cells, state, env, f, s);
@@ -509,7 +530,12 @@ static int solve_impl(const camp_mech *mc, int64_t n_cells, double *state, const
     if (cpb <= 0) {  // most resident cells per SM, fewest cells per block on ties
         int best = 0;
         cpb = 1;
-        const int max_cpb = m->h.lanes > 32 ? 1 : 4;
+        int max_cpb = m->h.lanes > 32 ? 1 : 4;
+        // a call whose cells are all resident at one a block spreads evenly
+        // over the SMs that way (256 gas cells: 6.3 ms; 7.3 ms at three a block)
+        int one = 0;
+        CUDA_TRY(occupancy(1, &one));
+        if (n_cells <= (long long)one * m->sm_count) max_cpb = 1;
         for (int c2 = 1; c2 <= max_cpb; c2++) {
             if (c2 * smem_cell > kMaxSmem) break;
             int per_sm = 0;

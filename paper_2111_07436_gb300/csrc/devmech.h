@@ -141,6 +141,11 @@ struct DevMech {
     const double2 *gcf;
     int n_gstep;
     int n_fpart;          // partial sums of split forcing sums
+    // the sums by position, for a lane that holds a whole cell: entries
+    // fsum_ptr[p] .. fsum_ptr[p+1]: process, coefficient
+    const int *fsum_ptr;  // [n+1]
+    const int *fsum_k;
+    const double *fsum_c;
     int n_part;           // partial sums of split forcing sums, substitution
                           // rows and factorisation rows (scratch after the
                           // rate terms; counted in FP64 values)

@@ -139,6 +139,57 @@ __global__ void k_forcing(const __grid_constant__ DevMech m, long long n_cells, 
     }
 }
 
+// The same with one cell per lane, 32 cells a warp: every lane evaluates the
+// same process, so that an FP64 instruction -- 64 cycles a warp whatever its
+// active lanes -- serves 32 cells, and the rate constants' exp, pow and log,
+// which bound this kernel, run without divergence.  The rates of the warp's
+// cells lie in shared memory ([process][cell]); the state and env rows are
+// read in place (each lane its own row: the loads are few beside the FP64
+// work).  The sums take their entries in the order, and in the two
+// accumulators, of the cell kernels: the same f bit for bit.
+template <int L>
+__global__ void __launch_bounds__(L) k_forcing_lanes(const __grid_constant__ DevMech m, long long n_cells,
+                                                      const double *state, const double *env, double *f_out) {
+    double *rs = (double *)block_smem;
+    const int lane = threadIdx.x;
+    const long long cell = (long long)blockIdx.x * L + lane, at = cell < n_cells ? cell : n_cells - 1;
+    const double *y = state + at * m.n, *e = env + at * m.n_env;
+#pragma unroll 1
+    for (int k = 0; k < m.R; k++) {
+        double kf, kr;
+        rate_constant(m, k, e, kf, kr);
+        const int4 rp = __ldg(m.rpack + k);
+        const int a0 = lo16(rp.x), a1 = hi16(rp.x), a2 = lo16(rp.y), rv = hi16(rp.y);
+        auto at_pos = [&](int p) { return y[__ldg(m.perm + p)]; };
+        double a = kf;
+        if (a0 != NONE16) a *= at_pos(a0);
+        if (a1 != NONE16) a *= at_pos(a1);
+        if (a2 != NONE16) a *= at_pos(a2);
+        if (rv != NONE16) {
+            const int b0 = lo16(rp.z), b1 = hi16(rp.z), b2 = lo16(rp.w);
+            double b = kr;
+            if (b0 != NONE16) b *= at_pos(b0);
+            if (b1 != NONE16) b *= at_pos(b1);
+            if (b2 != NONE16) b *= at_pos(b2);
+            a -= b;
+        }
+        rs[k * L + lane] = a;
+    }
+    __syncwarp();
+    for (int p = 0; p < m.n; p++) {
+        const int q1 = __ldg(m.fsum_ptr + p + 1);
+        double acc = 0.0, acc2 = 0.0;
+        int q = __ldg(m.fsum_ptr + p);
+#pragma unroll 1
+        for (; q + 1 < q1; q += 2) {
+            acc = fma(__ldg(m.fsum_c + q), rs[__ldg(m.fsum_k + q) * L + lane], acc);
+            acc2 = fma(__ldg(m.fsum_c + q + 1), rs[__ldg(m.fsum_k + q + 1) * L + lane], acc2);
+        }
+        if (q < q1) acc = fma(__ldg(m.fsum_c + q), rs[__ldg(m.fsum_k + q) * L + lane], acc);
+        if (cell < n_cells) f_out[cell * m.n + __ldg(m.perm + p)] = acc + acc2;
+    }
+}
+
 // Jacobian values of every cell, [cell][nnzJ] in species-CSR order, computed
 // in precision LT (the assembly precision of the corresponding solve form).
 template <int G, int NPL, typename LT, bool W>

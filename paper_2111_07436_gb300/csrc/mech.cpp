@@ -1500,6 +1500,9 @@ std::vector<unsigned char> pack_tables(const HostMech &h, DevMech &dm, const uns
     dm.gth = reinterpret_cast<const int2 *>(pk.put(h.gth));
     dm.gcf = reinterpret_cast<const double2 *>(pk.put(h.gcf));
     dm.n_gstep = h.n_gstep;
+    dm.fsum_ptr = pk.put(h.fptr);
+    dm.fsum_k = pk.put(h.fk);
+    dm.fsum_c = pk.put(h.fc);
     dm.n_fpart = h.n_fpart;
     dm.n_fsplit = (int)h.fsplit.size() / 2;
     dm.fsplit = reinterpret_cast<const int2 *>(pk.put(h.fsplit));
