@@ -32,6 +32,11 @@ namespace campdev {
 namespace cg = cooperative_groups;
 
 constexpr int ARROW_NT = 256;     // threads per CTA
+// CTAs an SM holds.  The particle loops are chains of loads and of FP64
+// instructions that one warp issues every 64 cycles, so warps count for more
+// than registers (10^4 particles, 152 cells, mixed / FP64 form: 2 CTAs 183 /
+// 236 ms, 3: 148 / 192, 4: 134 / 180, 5: 125 / 173, 6: 132 / 184).
+constexpr int ARROW_CTAS = 5;
 constexpr int ARROW_MAX_CL = 16;  // CTAs per cluster
 constexpr int ARROW_MAX_RG = 64;  // gas processes
 constexpr int ARROW_RED = CAMP_ARROW_MAX_C * CAMP_ARROW_MAX_C + 2;  // values of one reduction
@@ -246,47 +251,75 @@ __device__ inline bool arrow_particle_factor(const ArrowDev &a, int p, LT *lu, L
     return bad;
 }
 
-// Forward part for one particle: y_p = L^-1 b_p in xp (b_p given there),
-// and sum_p L_Gp y_p added to fw [n_c]
-template <typename LT>
-__device__ inline void arrow_particle_forward(const ArrowDev &a, int p, const LT *lu, LT *xp, double *fw) {
+// The particle's solves, its values in registers: NPM is a bound of n_phi
+// known to the compiler (8 or 16), so that the loops unroll and the loads of
+// the particle's LU block, which no value depends on, are all in flight
+// together; with runtime loops each waited for its own load (54% of the
+// kernel's stall samples).
+//
+// Forward part: y_p = L^-1 b_p in x (b_p given there), and sum_p L_Gp y_p
+// added to fw [n_c]
+template <int NPM, typename LT>
+__device__ __forceinline__ void arrow_particle_forward(const ArrowDev &a, int p, const LT *lu, LT (&x)[NPM], double *fw) {
     const int np = a.n_phi, nc = a.n_c;
     const size_t P = (size_t)a.P;
-    const LT *B = lu, *LGp = lu + (size_t)np * np * P + (size_t)np * nc * P;
-    LT y[CAMP_ARROW_MAX_PHI];
-    for (int i = 0; i < np; i++) {
-        LT s = xp[(size_t)i * P + p];
-        for (int j = 0; j < i; j++) s -= B[((size_t)i * np + j) * P + p] * y[j];
-        y[i] = s;
-        xp[(size_t)i * P + p] = s;
+    const LT *B = lu + p, *LGp = B + ((size_t)np * np + (size_t)np * nc) * P;
+#pragma unroll
+    for (int i = 1; i < NPM; i++) {
+        if (i < np) {
+            LT b[NPM];
+#pragma unroll
+            for (int j = 0; j < i; j++) b[j] = B[((size_t)i * np + j) * P];
+#pragma unroll
+            for (int j = 0; j < i; j++) x[i] -= b[j] * x[j];
+        }
     }
+#pragma unroll 2
     for (int c = 0; c < nc; c++) {
-        LT s = (LT)0;
-        for (int j = 0; j < np; j++) s += LGp[((size_t)c * np + j) * P + p] * y[j];
+        LT l[NPM], s = (LT)0;
+#pragma unroll
+        for (int j = 0; j < NPM; j++) l[j] = j < np ? LGp[((size_t)c * np + j) * P] : (LT)0;
+#pragma unroll
+        for (int j = 0; j < NPM; j++)
+            if (j < np) s += l[j] * x[j];
         fw[c] += from_lu(s);
     }
 }
 
-// Backward part for one particle: x_p = U^-1 (y_p - U_pG x_G) in xp
-template <typename LT>
-__device__ inline void arrow_particle_backward(const ArrowDev &a, int p, const LT *lu, LT *xp, const LT *xgas) {
+// Backward part: x_p = U^-1 (y_p - U_pG x_G) in x (y_p given there)
+template <int NPM, typename LT>
+__device__ __forceinline__ void arrow_particle_backward(const ArrowDev &a, int p, const LT *lu, LT (&x)[NPM],
+                                                        const LT *xgas) {
     const int np = a.n_phi, nc = a.n_c;
     const size_t P = (size_t)a.P;
-    const LT *B = lu, *UpG = lu + (size_t)np * np * P;
-    LT x[CAMP_ARROW_MAX_PHI];
-    for (int i = np - 1; i >= 0; i--) {
-        LT s = xp[(size_t)i * P + p];
-        for (int c = 0; c < nc; c++) s -= UpG[((size_t)i * nc + c) * P + p] * xgas[__ldg(a.coupled + c)];
-        for (int j = i + 1; j < np; j++) s -= B[((size_t)i * np + j) * P + p] * x[j];
-        x[i] = s * B[((size_t)i * np + i) * P + p];
-        xp[(size_t)i * P + p] = x[i];
+    const LT *B = lu + p, *UpG = B + (size_t)np * np * P;
+    for (int c = 0; c < nc; c++) {
+        const LT xg = xgas[__ldg(a.coupled + c)];
+        LT u[NPM];
+#pragma unroll
+        for (int i = 0; i < NPM; i++) u[i] = i < np ? UpG[((size_t)i * nc + c) * P] : (LT)0;
+#pragma unroll
+        for (int i = 0; i < NPM; i++)
+            if (i < np) x[i] -= u[i] * xg;
+    }
+#pragma unroll
+    for (int i = NPM - 1; i >= 0; i--) {
+        if (i < np) {
+            LT b[NPM];
+#pragma unroll
+            for (int j = i; j < NPM; j++) b[j] = j < np ? B[((size_t)i * np + j) * P] : (LT)0;
+#pragma unroll
+            for (int j = i + 1; j < NPM; j++)
+                if (j < np) x[i] -= b[j] * x[j];
+            x[i] *= b[i];
+        }
     }
 }
 
 // ---- one cell over [0, dt] ----------------------------------------------------
 // The step controller of integrate_cell (cellsolve.cuh), step for step, on
 // the block-arrow storage.  Returns the status (uniform over the cluster).
-template <typename LT>
+template <int NPM, typename LT>
 __device__ int arrow_integrate_cell(const DevMech &mt, const ArrowDev &a, ArrowSmem<LT> &sm,
                                     const cg::cluster_group &cl, char *scratch, double *__restrict__ y_cell,
                                     const double *__restrict__ env, double dt, double rtol,
@@ -500,11 +533,15 @@ __device__ int arrow_integrate_cell(const DevMech &mt, const ArrowDev &a, ArrowS
     auto rescale = [&](int q, double eta) {
         for (int p = lane; p < a.P; p += L)
             for (int i = 0; i < np; i++) {
-                double f = 1.0;
-                for (int j = 1; j <= q; j++) {
-                    f *= eta;
-                    Z(j, i, p) *= f;
-                }
+                double f = 1.0, zz[QMAX + 1];
+#pragma unroll
+                for (int j = 1; j <= QMAX; j++) zz[j] = j <= q ? Z(j, i, p) : 0.0;
+#pragma unroll
+                for (int j = 1; j <= QMAX; j++)
+                    if (j <= q) {
+                        f *= eta;
+                        Z(j, i, p) = zz[j] * f;
+                    }
             }
         if (gas_own) {
             double f = 1.0;
@@ -642,18 +679,37 @@ __device__ int arrow_integrate_cell(const DevMech &mt, const ArrowDev &a, ArrowS
                     double yl[ARROW_MAX_LOC], fl[ARROW_MAX_LOC];
                     int bad_f = 0;
                     for (int p = lane; p < a.P; p += L) {
-                        for (int i = 0; i < np; i++) yl[i] = Z(0, i, p);
-                        if (it)
-                            for (int i = 0; i < np; i++) yl[i] += E(i, p);
+                        double z1[NPM], ev[NPM];
+#pragma unroll
+                        for (int i = 0; i < NPM; i++) {
+                            ev[i] = 0.0;
+                            if (i < np) {
+                                yl[i] = Z(0, i, p);
+                                z1[i] = Z(1, i, p);
+                                if (it) ev[i] = E(i, p);
+                            }
+                        }
+                        if (it) {
+#pragma unroll
+                            for (int i = 0; i < NPM; i++)
+                                if (i < np) yl[i] += ev[i];
+                        }
                         for (int k = 0; k < nc; k++) yl[np + k] = sm.ygas[__ldg(a.coupled + k)];
                         arrow_particle_forcing(a, p, c.kfp, c.krp, yl, fl);
-                        for (int i = 0; i < np; i++) {
-                            bad_f += !finite_bits(fl[i]);
-                            const double r = fma(-gamma, fl[i], it ? E(i, p) : 0.0);
-                            X(i, p) = to_lu<LT>(-fma(Z(1, i, p), rl1, r));
+                        LT x[NPM];
+#pragma unroll
+                        for (int i = 0; i < NPM; i++) {
+                            x[i] = (LT)0;
+                            if (i < np) {
+                                bad_f += !finite_bits(fl[i]);
+                                x[i] = to_lu<LT>(-fma(z1[i], rl1, fma(-gamma, fl[i], ev[i])));
+                            }
                         }
                         for (int k = 0; k < nc; k++) part[k] += fl[np + k];
-                        arrow_particle_forward<LT>(a, p, c.lu, c.xp, part + nc);
+                        arrow_particle_forward<NPM, LT>(a, p, c.lu, x, part + nc);
+#pragma unroll
+                        for (int i = 0; i < NPM; i++)
+                            if (i < np) X(i, p) = x[i];
                     }
                     part[2 * nc] = (double)bad_f;
                     gas_rates();
@@ -695,17 +751,30 @@ __device__ int arrow_integrate_cell(const DevMech &mt, const ArrowDev &a, ArrowS
                     double s2[3] = {0.0, red[2 * nc] + gnf, 0.0};
                     int bad_x = 0;
                     for (int p = lane; p < a.P; p += L) {
-                        arrow_particle_backward<LT>(a, p, c.lu, c.xp, sm.xgas);
-                        for (int i = 0; i < np; i++) {
-                            LT xl = X(i, p) * scale;
-                            double en = from_lu(xl);
-                            const double wv = Wt(i, p);
-                            if (it) en += E(i, p);
-                            E(i, p) = en;
-                            s2[0] += from_lu(upd_term(xl, norm_weight<LT>(wv)));
-                            bad_x += !isfinite(xl);
-                            const double v = en * wv;
-                            s2[2] += v * v;
+                        LT x[NPM];
+                        double ev[NPM], wv[NPM];
+#pragma unroll
+                        for (int i = 0; i < NPM; i++) {
+                            x[i] = (LT)0;
+                            if (i < np) {
+                                x[i] = X(i, p);
+                                wv[i] = Wt(i, p);
+                                if (it) ev[i] = E(i, p);
+                            }
+                        }
+                        arrow_particle_backward<NPM, LT>(a, p, c.lu, x, sm.xgas);
+#pragma unroll
+                        for (int i = 0; i < NPM; i++) {
+                            if (i < np) {
+                                const LT xl = x[i] * scale;
+                                double en = from_lu(xl);
+                                if (it) en += ev[i];
+                                E(i, p) = en;
+                                s2[0] += from_lu(upd_term(xl, norm_weight<LT>(wv[i])));
+                                bad_x += !isfinite(xl);
+                                const double v = en * wv[i];
+                                s2[2] += v * v;
+                            }
                         }
                     }
                     if (gas_own) {
@@ -783,17 +852,30 @@ __device__ int arrow_integrate_cell(const DevMech &mt, const ArrowDev &a, ArrowS
         int bad_z = 0;
         for (int p = lane; p < a.P; p += L)
             for (int i = 0; i < np; i++) {
-                const double ev = E(i, p);
-                for (int j = 0; j <= q; j++) Z(j, i, p) += mt.lcoef[q][j] * ev;
-                bad_z += !finite_bits(Z(0, i, p));
+                // every load first: the stores below would hold the later ones back
+                const double ev = E(i, p), at = atol_of(species(i, p));
+                double zz[QMAX + 1], epv = 0.0, w = 0.0, zqv = 0.0;
+#pragma unroll
+                for (int j = 0; j <= QMAX; j++) zz[j] = j <= q ? Z(j, i, p) : 0.0;
                 if (select) {
-                    const double w = Wt(i, p);
-                    const double zq = Z(q, i, p) * w, de = (ev - EP(i, p)) * w;
+                    epv = EP(i, p);
+                    w = Wt(i, p);
+                }
+#pragma unroll
+                for (int j = 0; j <= QMAX; j++)
+                    if (j <= q) {
+                        zz[j] += mt.lcoef[q][j] * ev;
+                        Z(j, i, p) = zz[j];
+                        zqv = zz[j];
+                    }
+                bad_z += !finite_bits(zz[0]);
+                if (select) {
+                    const double zq = zqv * w, de = (ev - epv) * w;
                     acc[1] += zq * zq;
                     acc[2] += de * de;
                 }
                 EP(i, p) = ev;
-                Wt(i, p) = C::weight(rtol, Z(0, i, p), atol_of(species(i, p)));  // the next step's
+                Wt(i, p) = C::weight(rtol, zz[0], at);  // the next step's
             }
         if (gas_own) {
             for (int j = 0; j <= q; j++) zg[j] += mt.lcoef[q][j] * eg;

@@ -456,7 +456,7 @@ static int arrow_solve(camp_mech *m, int64_t n_cells, double *state, const doubl
     if (ncl == 0) {
         std::lock_guard<std::mutex> lk(m->mu);
         int n = 0;
-        CUDA_TRY(camp_arrow_max_clusters(lu, cl, &n));
+        CUDA_TRY(camp_arrow_max_clusters(m->ad, lu, cl, &n));
         if (n < 1) return fail(CAMP_E_UNSUPPORTED, "a block-arrow cluster does not fit on the device");
         ncl = n;
     }

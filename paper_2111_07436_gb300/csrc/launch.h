@@ -93,7 +93,7 @@ cudaError_t camp_launch_lu_solve_f64(const DevMech &m, long long n_cells, const 
 // of camp_arrow_cell_bytes each.
 #include "arrow.h"
 size_t camp_arrow_cell_bytes(const ArrowDev &a, int lu_elem);
-cudaError_t camp_arrow_max_clusters(int lu_elem, int cl_size, int *n);
+cudaError_t camp_arrow_max_clusters(const ArrowDev &a, int lu_elem, int cl_size, int *n);
 cudaError_t camp_arrow_launch(const DevMech &mt, const ArrowDev &a, const SolveArgs &s, int lu_elem, char *scratch,
                               size_t cell_bytes, int n_clusters, int cl_size, cudaStream_t st);
 cudaError_t camp_arrow_forcing(const DevMech &mt, const ArrowDev &a, long long n_cells, const double *state,

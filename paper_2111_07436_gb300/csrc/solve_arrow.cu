@@ -7,12 +7,13 @@ namespace campdev {
 
 // Every cell over one or more outer steps; clusters take cells round-robin
 // (cluster c: cells c, c + clusters, ...), each with its own slice of the
-// scratch.  Four CTAs per SM (64 registers a thread): the particle loops are
-// chains of dependent global loads, and the extra warps hide their latency
-// (measured at 10^4 particles: 2.0x one CTA per SM, 1.3x two).
-template <typename LT>
-__global__ void __launch_bounds__(ARROW_NT, 4)
-    k_arrow(DevMech mt, ArrowDev a, SolveArgs s, char *scratch, size_t cell_bytes) {
+// scratch.  NPM: the compiler's bound of the phase species per particle (8 up
+// to 8 species, else 16; with runtime loops instead the kernel took 148.5
+// against 124.9 ms on 152 cells of 10^4 particles, 7 species each).
+template <typename LT, int NPM>
+__global__ void __launch_bounds__(ARROW_NT, ARROW_CTAS)
+    k_arrow(const __grid_constant__ DevMech mt, const __grid_constant__ ArrowDev a, const __grid_constant__ SolveArgs s,
+            char *scratch, size_t cell_bytes) {
     __shared__ ArrowSmem<LT> sm;
     cg::cluster_group cl = cg::this_cluster();
     const long long csz = cl.num_blocks();
@@ -23,7 +24,7 @@ __global__ void __launch_bounds__(ARROW_NT, 4)
         CellStats st, tot{0, 0, 0, 0, 0};
         int status = ST_OK;
         for (int o = 0; o < s.n_outer && status == ST_OK; o++) {
-            status = arrow_integrate_cell<LT>(mt, a, sm, cl, mine, s.state + cell * a.n, s.env + cell * a.n_env,
+            status = arrow_integrate_cell<NPM, LT>(mt, a, sm, cl, mine, s.state + cell * a.n, s.env + cell * a.n_env,
                                               s.dt, s.rtol, s.atol, s.atol_len, s.max_steps, s.hmin_frac,
                                               s.step ? s.step + cell : nullptr, par, st,
                                               s.traj ? s.traj + ((long long)o * s.n_cells + cell) * a.n : nullptr);
@@ -106,10 +107,14 @@ __global__ void __launch_bounds__(ARROW_NT) k_arrow_forcing(DevMech mt, ArrowDev
 }  // namespace campdev
 
 namespace {
-template <typename LT>
-cudaError_t arrow_config(int cl_size, int n_clusters, cudaStream_t st, cudaLaunchConfig_t &cfg,
+// the kernel for an LU precision and a bound of the species per particle
+using ArrowKernel = void (*)(DevMech, ArrowDev, SolveArgs, char *, size_t);
+ArrowKernel arrow_kernel(int lu_elem, int n_phi) {
+    if (lu_elem == 4) return n_phi <= 8 ? campdev::k_arrow<float, 8> : campdev::k_arrow<float, 16>;
+    return n_phi <= 8 ? campdev::k_arrow<double, 8> : campdev::k_arrow<double, 16>;
+}
+cudaError_t arrow_config(ArrowKernel kern, int cl_size, int n_clusters, cudaStream_t st, cudaLaunchConfig_t &cfg,
                          cudaLaunchAttribute *attr) {
-    auto kern = campdev::k_arrow<LT>;
     if (cl_size > 8) {
         cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
         if (e != cudaSuccess) return e;
@@ -131,29 +136,23 @@ cudaError_t arrow_config(int cl_size, int n_clusters, cudaStream_t st, cudaLaunc
 
 size_t camp_arrow_cell_bytes(const ArrowDev &a, int lu_elem) { return campdev::arrow_cell_bytes(a, lu_elem); }
 
-cudaError_t camp_arrow_max_clusters(int lu_elem, int cl_size, int *n) {
+cudaError_t camp_arrow_max_clusters(const ArrowDev &a, int lu_elem, int cl_size, int *n) {
+    const ArrowKernel kern = arrow_kernel(lu_elem, a.n_phi);
     cudaLaunchConfig_t cfg;
     cudaLaunchAttribute attr[1];
-    cudaError_t e = lu_elem == 4 ? arrow_config<float>(cl_size, 1, nullptr, cfg, attr)
-                                 : arrow_config<double>(cl_size, 1, nullptr, cfg, attr);
+    cudaError_t e = arrow_config(kern, cl_size, 1, nullptr, cfg, attr);
     if (e != cudaSuccess) return e;
-    return lu_elem == 4 ? cudaOccupancyMaxActiveClusters(n, campdev::k_arrow<float>, &cfg)
-                        : cudaOccupancyMaxActiveClusters(n, campdev::k_arrow<double>, &cfg);
+    return cudaOccupancyMaxActiveClusters(n, kern, &cfg);
 }
 
 cudaError_t camp_arrow_launch(const DevMech &mt, const ArrowDev &a, const SolveArgs &s, int lu_elem, char *scratch,
                               size_t cell_bytes, int n_clusters, int cl_size, cudaStream_t st) {
+    const ArrowKernel kern = arrow_kernel(lu_elem, a.n_phi);
     cudaLaunchConfig_t cfg;
     cudaLaunchAttribute attr[1];
-    cudaError_t e;
-    if (lu_elem == 4) {
-        e = arrow_config<float>(cl_size, n_clusters, st, cfg, attr);
-        if (e == cudaSuccess) e = cudaLaunchKernelEx(&cfg, campdev::k_arrow<float>, mt, a, s, scratch, cell_bytes);
-    } else {
-        e = arrow_config<double>(cl_size, n_clusters, st, cfg, attr);
-        if (e == cudaSuccess) e = cudaLaunchKernelEx(&cfg, campdev::k_arrow<double>, mt, a, s, scratch, cell_bytes);
-    }
-    return e;
+    cudaError_t e = arrow_config(kern, cl_size, n_clusters, st, cfg, attr);
+    if (e != cudaSuccess) return e;
+    return cudaLaunchKernelEx(&cfg, kern, mt, a, s, scratch, cell_bytes);
 }
 
 cudaError_t camp_arrow_forcing(const DevMech &mt, const ArrowDev &a, long long n_cells, const double *state,
