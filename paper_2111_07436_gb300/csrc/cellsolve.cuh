@@ -352,6 +352,7 @@ template <int G>
 __device__ __forceinline__ void rate_terms(const DevMech &m, const double *ys, const double *kfs, const double *kr,
                                            double *rs, int lane) {
     const int R = m.R;
+    if (R == 0) return;
     auto at = [&](int p) { return ys[p != NONE16 ? p : 0]; };
     int k = min(lane, R - 1);
     int4 rp = __ldg(m.rpack + k);
@@ -599,7 +600,7 @@ __device__ __forceinline__ void eval_f_ys(const DevMech &m, const CellPtr<LT> &c
     if constexpr (W) {
         water_update<G>(m, c.pw, c.ys, lane, gm);
         const double *invl = pw_invl(m, c.pw);
-        int4 rp = __ldg(m.rpack + min(lane, m.R - 1));
+        int4 rp = __ldg(m.rpack + max(min(lane, m.R - 1), 0));
 #pragma unroll 1
         for (int k = lane; k < m.R; k += G) {
             const int4 rn = __ldg(m.rpack + min(k + G, m.R - 1));

@@ -22,14 +22,23 @@ __device__ __forceinline__ unsigned group_mask() {
 // The whole solve: each group of G lanes integrates one cell at a time.  With
 // `queue` null the mapping is static (cell = block * cpb + group); otherwise
 // the groups take cells from the counter until it passes n_cells.
-// Register caps: the FP32-LU form with one-warp cells is limited by
-// registers and shared memory together (168 a lane fits 12 cells per SM;
-// 224 fits 9); 64-thread cells with 4 slots take 168 in both forms
-// (measured: FP32-LU 6 cells per SM, faster than 128 with spills or 225
-// without a cap; FP64 form 7% faster than with 200); 128-thread cells take
-// 168 in the FP64 form (3 cells per SM instead of 2: 7% faster despite
-// spills; the FP32-LU form gains nothing); the FP64 form and the other
-// block cells may take the architectural maximum.
+// Register caps: the FP32-LU form with one-warp cells takes 168 a lane, the
+// most that leaves three warps to each of an SM's four sub-partitions (12
+// cells; 184 to 232 leave two, 8 cells: 62 -> 69 ms for 16384 gas-72 cells,
+// though a lone cell is 15% faster without the spills); 64-thread cells with
+// 4 slots take 168 in both forms (6 cells per SM; 200, five cells, 40.8 ->
+// 42.7 ms for 4096 multiphase-232 cells); 128-thread cells take 168 in the
+// FP64 form (3 cells per SM instead of 2: 7% faster despite spills; the
+// FP32-LU form gains nothing); the FP64 form and the other block cells may
+// take the architectural maximum.
+//
+// What bounds it: a cell is one dependent chain (about 4700 instructions a
+// Newton iteration of a gas-72 cell, 115 of them FP64 at 64 cycles each), so
+// a lone warp takes 25k cycles an iteration and 12 of them an SM 40k: of the
+// issue slots 34% are used, and a warp waits on fixed latencies and the FP64
+// port (24%), shared memory and shuffles (23%), instruction fetch (16%; the
+// loop, the setup and the step code exceed the 32 KB of first-level
+// instruction cache) and table loads (11%; 28 KB of L1 beside 12 cells).
 template <int G, int NPL, typename LT, bool W>
 __global__ void __maxnreg__((G == 64 && NPL == 4) || (G == 128 && sizeof(LT) == 8) ? 168
                             : ((sizeof(LT) == 8 || G > 32) ? 255 : (NPL >= 6 ? 224 : 168)))

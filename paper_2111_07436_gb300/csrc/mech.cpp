@@ -249,6 +249,10 @@ static int electrolyte_species(const HostMech &h, int b, int e) {
     return h.n_gas + b * n_phase + h.el_phase[e];
 }
 
+// Partial slots one level may use (FP64 values of per-cell shared memory):
+// a longer chunk length is taken when the level's splits would need more.
+static const long long kLevelPartials = 2048;
+
 // ---- integer structure -----------------------------------------------------
 static std::vector<int> dependence(const Process &p) {  // species entering r_k
     std::vector<int> d;
@@ -560,9 +564,6 @@ static RowSplit split_row(const std::vector<uint32_t> &ops, int CH) {
     return rs;
 }
 
-// Partial slots one level may use (FP64 values of per-cell shared memory):
-// a longer chunk length is taken when the level's splits would need more.
-static const long long kLevelPartials = 2048;
 
 static const uint32_t kFactorNop = CAMP_OP_DIV | ((uint32_t)CAMP_OP_NOSRC << 16);
 
@@ -840,8 +841,8 @@ static void build_tables(HostMech &h) {
     };
     {
         const int compact = stored(h.d, (n - h.d) | 1);
-        // partials and the water parameter's values at most, besides the LU
-        const int scratch = 3 * 2048 + 4 * n;
+        // a bound of the partial sums and the water parameter's values
+        const int scratch = (int)kLevelPartials + n;
         auto bytes = [&](int nlu, int elem) { return cell_smem(n, R, h.n_rev, nlu, elem, scratch, 1 << 20, 0, 0, h.lanes).bytes; };
         auto fits = [&](int d) {
             const int s = stored(d, stride(n - d));
