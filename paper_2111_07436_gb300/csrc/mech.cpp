@@ -753,9 +753,10 @@ static void build_tables(HostMech &h) {
         for (auto &e : fl[p]) { h.fk.push_back(e.first); h.fc.push_back(e.second); }
         h.fptr.push_back((int)h.fk.size());
     }
-    // the per-position sums over the lanes of one cell, longest processing
-    // time first; a sum longer than the lanes' mean load is cut into chunks
-    // whose partial sums a second pass adds in a fixed order
+    // the per-position sums over the lanes of one cell, first fit in order of
+    // length (the read lists run as long as the fullest lane's); a sum longer
+    // than the lanes' mean load is cut into chunks whose partial sums a second
+    // pass adds in a fixed order
     {
         const int NL = h.lanes;
         long long total = 0;
