@@ -10,12 +10,6 @@
 #include <stdint.h>
 #include <vector_types.h>
 
-#ifdef __CUDACC__
-#define CAMP_HD __host__ __device__
-#else
-#define CAMP_HD
-#endif
-
 #define CAMP_QMAX 5
 #define CAMP_MAXFAC 3  // at most 3 factors (with multiplicity) per rate term
 
@@ -68,6 +62,38 @@ inline int camp_alt_lanes(int n) {
 // group's static reduction scratch).
 constexpr int CAMP_MAX_SMEM = 227 * 1024 - 256;
 
+// Register slots a lane of an n-species cell (the water builds hold one
+// one-warp shape)
+inline int camp_cell_slots(int n, int lanes, bool water) {
+    if (lanes == 32 && !water) {
+        const int need = (n + 31) / 32;
+        return need <= 4 ? need : need <= 6 ? 6 : 8;
+    }
+    return lanes == 64 && n <= 256 ? 4 : 8;
+}
+
+// Registers a lane of the solve kernel (kernels.cuh has the reasons)
+constexpr int camp_solve_regs(int lanes, int slots, int lu_elem) {
+    return (lanes == 64 && slots == 4) || (lanes == 128 && lu_elem == 8) ? 168
+           : lu_elem == 8 || lanes > 32                                  ? 255
+                                                                         : (slots >= 6 ? 224 : 168);
+}
+
+// Cells of `bytes` of shared memory that an SM holds, at the best cells per
+// block: 228 KB less 1 KB a block (and a block group's reduction scratch), and
+// whole warps to each of four register files of 16384, 256 at a time.
+inline int camp_resident_cells(int bytes, int n, int lanes, bool water, int lu_elem) {
+    const int regs = (camp_solve_regs(lanes, camp_cell_slots(n, lanes, water), lu_elem) * 32 + 255) & ~255;
+    const int warps = 4 * (16384 / regs), fixed = 1024 + (lanes > 32 ? 256 : 0);
+    int best = 0;
+    for (int c = 1; c <= (lanes == 32 ? 4 : 1) && c * bytes <= CAMP_MAX_SMEM; c++) {
+        const int by_smem = 228 * 1024 / (c * bytes + fixed), by_regs = warps / (c * lanes / 32);
+        const int cells = c * (by_smem < by_regs ? by_smem : by_regs);
+        if (cells > best) best = cells;
+    }
+    return best;
+}
+
 // Shared-memory layout of one cell (byte offsets).  rs holds the R rate
 // terms, then n_part partial sums (of split forcing sums inside an f
 // evaluation, of split substitution and factorisation rows inside a solve);
@@ -75,14 +101,16 @@ constexpr int CAMP_MAX_SMEM = 227 * 1024 - 256;
 // the FP64 form; none without one); fb the odd halves of the
 // forcing sums (n + n_fpart doubles), which saves FP64 adds where a lane owns
 // few positions: one-warp cells and block cells of up to 4 positions a lane.
-// Other cells, and a cell that only fits without it, have none (fb = -1) and
-// add the two halves of a sum where the sum ends.
+// Other cells, and a mechanism of which an SM holds more cells without it, have
+// none (fb = -1) and add the two halves of a sum where the sum ends (117
+// species, FP64: 2 cells an SM with it, 189 ms for 2048 cells; 3 without,
+// 143 ms).
 struct CellSmem {
     int ys, rs, kf, kr, pw, x, lu, fb, bytes;
 };
-CAMP_HD inline int camp_align16(int b) { return (b + 15) & ~15; }
-CAMP_HD inline CellSmem cell_smem(int n, int R, int n_rev, int nlu, int lu_elem, int n_part, int n_fpart, int n_pw,
-                                  int n_pw64, int lanes) {
+inline int camp_align16(int b) { return (b + 15) & ~15; }
+inline CellSmem cell_smem(int n, int R, int n_rev, int nlu, int lu_elem, int n_part, int n_fpart, int n_pw, int n_pw64,
+                          int lanes) {
     CellSmem c;
     int o = 0;
     c.ys = o; o = camp_align16(o + 8 * n);
@@ -102,7 +130,9 @@ CAMP_HD inline CellSmem cell_smem(int n, int R, int n_rev, int nlu, int lu_elem,
     }
     c.lu = o; o = camp_align16(o + lu_elem * nlu);
     const int with = camp_align16(o + 8 * (n + n_fpart));
-    c.fb = with <= CAMP_MAX_SMEM && n <= (lanes == 32 ? 8 : 4) * lanes ? o : -1;
+    const bool few = n <= (lanes == 32 ? 8 : 4) * lanes;
+    auto cells = [&](int bytes) { return camp_resident_cells(bytes, n, lanes, n_pw > 0, lu_elem); };
+    c.fb = few && with <= CAMP_MAX_SMEM && cells(with) >= cells(o) ? o : -1;
     c.bytes = c.fb >= 0 ? with : o;
     return c;
 }
@@ -170,7 +200,7 @@ struct DevMech {
     int nlu;              // storage entries
     int d;                // first position of the dense block (= n when there is none)
     int D;                // dense block size n - d
-    int LD;           // dense block row stride, 4 mod 8
+    int LD;               // dense block row stride, 4 mod 8
     int dbase;            // storage offset of the dense block
 
     // factorisation of the sparse part: row-wise (up-looking) ops, level by

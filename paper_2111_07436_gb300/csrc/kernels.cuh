@@ -40,8 +40,7 @@ __device__ __forceinline__ unsigned group_mask() {
 // loop, the setup and the step code exceed the 32 KB of first-level
 // instruction cache) and table loads (11%; 28 KB of L1 beside 12 cells).
 template <int G, int NPL, typename LT, bool W>
-__global__ void __maxnreg__((G == 64 && NPL == 4) || (G == 128 && sizeof(LT) == 8) ? 168
-                            : ((sizeof(LT) == 8 || G > 32) ? 255 : (NPL >= 6 ? 224 : 168)))
+__global__ void __maxnreg__(camp_solve_regs(G, NPL, (int)sizeof(LT)))
     k_solve(const __grid_constant__ DevMech m, const __grid_constant__ SolveArgs a) {
     const int group = threadIdx.x / G, lane = threadIdx.x % G;
     const unsigned gm = group_mask<G>();
