@@ -16,7 +16,7 @@
 
 struct camp_mech {
     camp::HostMech h;
-    DevMech dm;
+    DevMech dm, dm64;          // for the kernels with an FP32 and with an FP64 LU
     void *dev_tables = nullptr;
     int device = 0;
     int sm_count = 0;
@@ -218,14 +218,15 @@ static int mech_build(const char *json, size_t len, camp_mech **out, char *err, 
         delete m;
         return report(CAMP_E_UNSUPPORTED, "more than 2048 species");
     }
-    DevMech probe{};
-    std::vector<unsigned char> img = camp::pack_tables(m->h, probe, nullptr);
+    DevMech probe{}, probe64{};
+    std::vector<unsigned char> img = camp::pack_tables(m->h, probe, probe64, nullptr);
     if (camp_cell_smem_bytes(probe, 4) > kMaxSmem) {
         delete m;
         return report(CAMP_E_UNSUPPORTED, "per-cell working set exceeds shared memory");
     }
     if (!upload) {
         m->dm = probe;
+        m->dm64 = probe64;
         *out = m;
         g_err.clear();
         return CAMP_OK;
@@ -234,7 +235,7 @@ static int mech_build(const char *json, size_t len, camp_mech **out, char *err, 
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&m->sm_count, cudaDevAttrMultiProcessorCount, m->device);
     if (e == cudaSuccess) e = cudaMalloc(&m->dev_tables, img.size());
     if (e == cudaSuccess) {
-        img = camp::pack_tables(m->h, m->dm, (const unsigned char *)m->dev_tables);
+        img = camp::pack_tables(m->h, m->dm, m->dm64, (const unsigned char *)m->dev_tables);
         e = cudaMemcpy(m->dev_tables, img.data(), img.size(), cudaMemcpyHostToDevice);
     }
     if (e == cudaSuccess && m->arrow) {
@@ -272,14 +273,14 @@ static int mech_relane(camp_mech *m, int lanes) {
         return fail(CAMP_E_PARSE, e.what());
     }
     if (camp_pick_shape(h2.n, h2.lanes) < 0) return fail(CAMP_E_UNSUPPORTED, "no cell shape for this lane count");
-    DevMech probe{};
-    std::vector<unsigned char> img = camp::pack_tables(h2, probe, nullptr);
+    DevMech probe{}, probe64{};
+    std::vector<unsigned char> img = camp::pack_tables(h2, probe, probe64, nullptr);
     if (camp_cell_smem_bytes(probe, 4) > kMaxSmem)
         return fail(CAMP_E_UNSUPPORTED, "per-cell working set exceeds shared memory");
     void *tables = nullptr;
     CUDA_TRY(cudaMalloc(&tables, img.size()));
-    DevMech dm2{};
-    img = camp::pack_tables(h2, dm2, (const unsigned char *)tables);
+    DevMech dm2{}, dm264{};
+    img = camp::pack_tables(h2, dm2, dm264, (const unsigned char *)tables);
     const cudaError_t e = cudaMemcpy(tables, img.data(), img.size(), cudaMemcpyHostToDevice);
     if (e != cudaSuccess) {
         cudaFree(tables);
@@ -289,6 +290,7 @@ static int mech_relane(camp_mech *m, int lanes) {
     m->dev_tables = tables;
     m->h = std::move(h2);
     m->dm = dm2;
+    m->dm64 = dm264;
     std::memset(m->occ, 0, sizeof m->occ);
     return CAMP_OK;
 }
@@ -341,7 +343,7 @@ int camp_mech_info_get(const camp_mech *m, camp_mech_info *o) {
     o->nnz_lu = (int32_t)h.lu_colidx.size();
     o->rxn_map_len = (int32_t)h.rxn_map.size();
     o->dense_block = h.D;
-    o->lu_storage = h.nlu;
+    o->lu_storage = m->dm.nlu;
     o->smem_per_cell_mixed = camp_cell_smem_bytes(m->dm, 4);
     o->smem_per_cell_fp64 = camp_cell_smem_bytes(m->dm, 8);
     o->factor_updates = h.factor_updates;
@@ -519,7 +521,7 @@ static int solve_impl(const camp_mech *mc, int64_t n_cells, double *state, const
         if (m->occ[o.variant][cpb_] == 0) {
             const bool w = m->dm.n_wsec > 0;
             cudaError_t e = f32 ? (w ? camp_occupancy_f32w(m->dm, cpb_, per_sm) : camp_occupancy_f32(m->dm, cpb_, per_sm))
-                                : (w ? camp_occupancy_f64w(m->dm, cpb_, per_sm) : camp_occupancy_f64(m->dm, cpb_, per_sm));
+                                : (w ? camp_occupancy_f64w(m->dm64, cpb_, per_sm) : camp_occupancy_f64(m->dm64, cpb_, per_sm));
             if (e != cudaSuccess) return e;
             m->occ[o.variant][cpb_] = *per_sm > 0 ? *per_sm : -1;
         }
@@ -587,9 +589,9 @@ static int solve_impl(const camp_mech *mc, int64_t n_cells, double *state, const
         if (grid > 0x7fffffffLL) return fail(CAMP_E_INVAL, "too many cells for one launch");
     }
     if (m->dm.n_wsec > 0)
-        CUDA_TRY(f32 ? camp_launch_solve_f32w(m->dm, a, (int)grid, s) : camp_launch_solve_f64w(m->dm, a, (int)grid, s));
+        CUDA_TRY(f32 ? camp_launch_solve_f32w(m->dm, a, (int)grid, s) : camp_launch_solve_f64w(m->dm64, a, (int)grid, s));
     else
-        CUDA_TRY(f32 ? camp_launch_solve_f32(m->dm, a, (int)grid, s) : camp_launch_solve_f64(m->dm, a, (int)grid, s));
+        CUDA_TRY(f32 ? camp_launch_solve_f32(m->dm, a, (int)grid, s) : camp_launch_solve_f64(m->dm64, a, (int)grid, s));
     return CAMP_OK;
 }
 
@@ -905,7 +907,7 @@ int camp_forcing(const camp_mech *m, int64_t n_cells, const double *state, const
         CUDA_TRY(camp_arrow_forcing(m->dm, m->ad, n_cells, state, env, f, (cudaStream_t)stream));
         return CAMP_OK;
     }
-    CUDA_TRY(camp_launch_forcing(m->dm, n_cells, state, env, f, (cudaStream_t)stream));
+    CUDA_TRY(camp_launch_forcing(m->dm64, n_cells, state, env, f, (cudaStream_t)stream));
     return CAMP_OK;
 }
 
@@ -920,10 +922,10 @@ int camp_jacobian(const camp_mech *m, int64_t n_cells, const double *state, cons
     cudaStream_t s = (cudaStream_t)stream;
     if (m->dm.n_wsec > 0)
         CUDA_TRY(variant == CAMP_VARIANT_MIXED ? camp_launch_jacobian_f32w(m->dm, n_cells, state, env, jac, s)
-                                               : camp_launch_jacobian_f64w(m->dm, n_cells, state, env, jac, s));
+                                               : camp_launch_jacobian_f64w(m->dm64, n_cells, state, env, jac, s));
     else
         CUDA_TRY(variant == CAMP_VARIANT_MIXED ? camp_launch_jacobian_f32(m->dm, n_cells, state, env, jac, s)
-                                               : camp_launch_jacobian_f64(m->dm, n_cells, state, env, jac, s));
+                                               : camp_launch_jacobian_f64(m->dm64, n_cells, state, env, jac, s));
     return CAMP_OK;
 }
 
@@ -941,11 +943,11 @@ int camp_lu_solve(const camp_mech *m, int64_t n_cells, const double *state, cons
     if (m->dm.n_wsec > 0)
         CUDA_TRY(variant == CAMP_VARIANT_MIXED
                      ? camp_launch_lu_solve_f32w(m->dm, n_cells, state, env, gamma, b, x, status, s)
-                     : camp_launch_lu_solve_f64w(m->dm, n_cells, state, env, gamma, b, x, status, s));
+                     : camp_launch_lu_solve_f64w(m->dm64, n_cells, state, env, gamma, b, x, status, s));
     else
         CUDA_TRY(variant == CAMP_VARIANT_MIXED
                      ? camp_launch_lu_solve_f32(m->dm, n_cells, state, env, gamma, b, x, status, s)
-                     : camp_launch_lu_solve_f64(m->dm, n_cells, state, env, gamma, b, x, status, s));
+                     : camp_launch_lu_solve_f64(m->dm64, n_cells, state, env, gamma, b, x, status, s));
     return CAMP_OK;
 }
 

@@ -871,8 +871,9 @@ template <> struct Vec16<double> {
 // rows right of the panel are forward-substituted with the panel's unit lower
 // triangle (lane l takes columns l + 32 s); (3) one rank-DENSE_W update of
 // the trailing rows, 16 bytes of a row at a time, the multipliers already in
-// registers and the pivot rows broadcast.  The row stride is 4 mod 8 values,
-// so that 16-byte accesses of FP32 rows spread over all banks.  Every entry
+// registers and the pivot rows broadcast.  The row stride is 4 mod 8 FP32 or
+// 2 mod 4 FP64 values where that costs no resident cells (choose_strides), so
+// that 16-byte accesses of the rows spread over all banks.  Every entry
 // takes its updates one by one in pivot order, as a plain elimination does.
 // Pivots are checked and replaced by their reciprocals.
 constexpr int DENSE_W = 8;

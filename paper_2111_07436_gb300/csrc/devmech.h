@@ -197,10 +197,11 @@ struct DevMech {
     int n_jstep[8];
 
     // --- LU storage: sparse rows [0, nsp) then a dense trailing block ---
-    int nlu;              // storage entries
+    int nlu;              // storage entries (this form's: an FP32 or an FP64 LU)
     int d;                // first position of the dense block (= n when there is none)
     int D;                // dense block size n - d
-    int LD;               // dense block row stride, 4 mod 8
+    int LD;               // dense block row stride of this form (jls, fst, lops,
+                          // lred_off and ch hold offsets that follow it)
     int dbase;            // storage offset of the dense block
 
     // factorisation of the sparse part: row-wise (up-looking) ops, level by

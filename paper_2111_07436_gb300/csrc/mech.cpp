@@ -711,7 +711,8 @@ static void subst_passes(HostMech &h, const std::vector<SubstJob> &jobs, const s
 }
 
 // ---- device tables -----------------------------------------------------------
-static void build_tables(HostMech &h) {
+// `later`: rows by which the dense block starts later than it could
+static void build_tables(HostMech &h, int later) {
     const int n = h.n, R = (int)h.procs.size();
     const auto &ip = h.iperm;
 
@@ -829,34 +830,11 @@ static void build_tables(HostMech &h) {
         if ((double)cnt >= 0.75 * (double)(n - d) * (double)(n - d)) { h.d = d; break; }
     }
     if (n - h.d > 128) h.d = n - 128;  // the substitution keeps at most 4 block rows per lane
-    // The block's rows are padded to a stride of 4 mod 8 values (16-byte row
-    // pieces without bank conflicts).  Where that padding would take a
-    // mechanism over a limit that compact rows respect, the block shrinks
-    // until it does not.
-    auto stride = [](int D) { return D > 0 ? ((D + 3) & ~7) + 4 : 0; };
-    auto stored = [&](int d, int LD) {  // LU values stored with the block starting at d
-        int sp = 0;
-        for (int i = 0; i < n; i++)
-            for (int q = h.lu_rowptr[i]; q < h.lu_rowptr[i + 1]; q++) sp += (i < d || h.lu_colidx[q] < d);
-        return ((sp + 3) & ~3) + (n - d) * LD;
-    };
-    {
-        const int compact = stored(h.d, (n - h.d) | 1);
-        // a bound of the partial sums and the water parameter's values
-        const int scratch = (int)kLevelPartials + n;
-        auto bytes = [&](int nlu, int elem) { return cell_smem(n, R, h.n_rev, nlu, elem, scratch, 1 << 20, 0, 0, h.lanes).bytes; };
-        auto fits = [&](int d) {
-            const int s = stored(d, stride(n - d));
-            if (s <= compact) return true;
-            return s <= 32767 && bytes(s, 4) <= CAMP_MAX_SMEM &&
-                   (bytes(s, 8) <= CAMP_MAX_SMEM || cell_smem(n, R, h.n_rev, compact, 8, 0, 1 << 20, 0, 0, h.lanes).bytes > CAMP_MAX_SMEM);
-        };
-        while (h.d < n && !fits(h.d)) h.d++;
-    }
+    h.d = std::min(n, h.d + later);
     h.D = n - h.d;
-    h.LD = stride(h.D);
 
-    // storage offsets: sparse rows < d, the L21 part of rows >= d, then the block
+    // storage offsets: sparse rows < d, the L21 part of rows >= d, then the
+    // block with rows of D values (lu_offset gives a form's own)
     std::vector<int> lu_off(h.lu_colidx.size(), -1);
     int nsp = 0;
     for (int i = 0; i < n; i++)
@@ -865,8 +843,8 @@ static void build_tables(HostMech &h) {
     h.dbase = (nsp + 3) & ~3;
     for (int i = h.d; i < n; i++)
         for (int q = h.lu_rowptr[i]; q < h.lu_rowptr[i + 1]; q++)
-            if (h.lu_colidx[q] >= h.d) lu_off[q] = h.dbase + (i - h.d) * h.LD + (h.lu_colidx[q] - h.d);
-    h.nlu = h.dbase + h.D * h.LD;
+            if (h.lu_colidx[q] >= h.d) lu_off[q] = h.dbase + (i - h.d) * h.D + (h.lu_colidx[q] - h.d);
+    h.nlu = h.dbase + h.D * h.D;
     if (h.nlu > 32767) throw std::runtime_error("LU storage too large for the packed tables (32767 values)");
     auto off = [&](int i, int j) {
         auto b = h.lu_colidx.begin() + h.lu_rowptr[i], e = h.lu_colidx.begin() + h.lu_rowptr[i + 1];
@@ -1161,6 +1139,17 @@ static void build_tables(HostMech &h) {
     h.sub_pass.insert(h.sub_pass.end(), 4 * (size_t)h.lanes, -1);
 }
 
+// Storage offset of a table entry in the FP32 (f = 0) or FP64 (1) form
+static int lu_offset(const HostMech &h, int f, int o) {
+    const int q = o - h.dbase;
+    return h.D == 0 || q < 0 ? o : h.dbase + q / h.D * h.LD[f] + q % h.D;
+}
+static int form_nlu(const HostMech &h, int stride) { return h.dbase + h.D * stride; }
+static CellSmem form_smem(const HostMech &h, int f, int nlu) {
+    return cell_smem(h.n, (int)h.procs.size(), h.n_rev, nlu, f ? 8 : 4, std::max(std::max(h.n_fpart, h.n_spart), h.n_lpart),
+                     h.n_fpart, h.n_pw, h.n_pw64, h.lanes);
+}
+
 // Bounds of every index the device tables hold, checked once per mechanism
 // on the host: the kernels index shared memory and the tables with these
 // values unchecked, so an out-of-range entry is a compiler bug caught here
@@ -1232,8 +1221,9 @@ static void validate_tables(const HostMech &h) {
         if (!in(r[2] & 0xffff, 0, nlu) || !in(t, 0, nnzJ)) fail("jls target");
     }
     // LU: storage layout, factorisation jobs, substitution lists
-    if (h.dbase + h.D * h.LD > nlu || h.d + h.D != n || h.D > 128) fail("dense block");
-    if (h.D > 0 && (h.LD < h.D || h.LD % 8 != 4 || h.dbase % 4 != 0)) fail("dense block alignment");
+    if (h.dbase + h.D * h.D > nlu || h.d + h.D != n || h.D > 128) fail("dense block");
+    if (h.D > 0 && (h.LD[0] < h.D || h.LD[1] < h.D || h.LD[0] % 4 || h.LD[1] % 2 || h.dbase % 4)) fail("dense block alignment");
+    if (form_nlu(h, h.LD[0]) > 32767 || form_nlu(h, h.LD[1]) > 32767) fail("dense block size");
     for (int i = 0; i < h.d; i++) if (!in(h.udiag[i], 0, nlu)) fail("udiag");
     const int nops = (int)h.lops.size();
     if (h.fst.size() != ((size_t)h.fst_ptr.back() + 1) * h.lanes || h.fst_part.size() + 1 != h.fst_ptr.size()) fail("fst size");
@@ -1314,19 +1304,47 @@ static void validate_tables(const HostMech &h) {
         if (h.su_ptr[i] > h.su_ptr[i + 1] || h.sl_ptr[i] > h.sl_ptr[i + 1]) fail("substitution pointers");
 }
 
+// The dense block's row stride of each form.  16-byte accesses need a
+// multiple of 4 FP32 or 2 FP64 values, and spread over all banks at 4 mod 8
+// or 2 mod 4.  The plain multiple is taken where that padding costs resident
+// cells (4096 FP32 cells of 80 rows: 7 an SM at stride 80, 35.7 ms; 6 at 84,
+// 37.0 ms), but not at 128 bytes mod 128, where every row starts in the same
+// bank (FP32, 61 rows: 11 cells at stride 64, 39.7 ms; 10 at 68, 34.3 ms;
+// FP64, 63 rows: 6 at 64, 111 ms; 5 at 66, 103 ms) unless it keeps twice the
+// cells.  False if a form fits the device with compact rows but not with the
+// multiple: the block then has to start later.
+static bool choose_strides(HostMech &h) {
+    const int D = h.D;
+    auto cells = [&](int f, int stride) {
+        const int nlu = form_nlu(h, stride);
+        return nlu > 32767 ? 0 : camp_resident_cells(form_smem(h, f, nlu).bytes, h.n, h.lanes, !h.el_phase.empty(), f ? 8 : 4);
+    };
+    for (int f = 0; f < 2; f++) {
+        const int m = f ? 2 : 4, multiple = (D + m - 1) / m * m, spread = multiple % (2 * m) ? multiple : multiple + m;
+        const int a = cells(f, spread), b = cells(f, multiple);
+        const bool one_bank = multiple % (8 * m) == 0;
+        h.LD[f] = D == 0 ? 0 : a == 0 || (b > a && (!one_bank || b >= 2 * a)) ? multiple : spread;
+        if (D > 0 && cells(f, h.LD[f]) == 0 && (cells(f, D | 1) > 0 || form_nlu(h, h.LD[f]) > 32767)) return false;
+    }
+    return true;
+}
+
 HostMech compile_mechanism(const char *json, size_t len, int instances, int lanes) {
     Value root = campjson::parse(json, len);
-    HostMech h;
-    read_processes(root, h, instances);
-    if (h.n < 1) throw std::runtime_error("mechanism has no species");
-    h.lanes = lanes > 0 ? lanes : camp_cell_lanes(h.n);
-    if ((h.lanes != 32 && h.lanes != 64 && h.lanes != 128 && h.lanes != 256) || h.n > 8 * h.lanes)
-        throw std::runtime_error("lanes per cell must be 32, 64, 128 or 256, with at most 8 species a lane");
-    build_structure(h);
-    build_tables(h);
-    pack_records(h);
-    validate_tables(h);
-    return h;
+    for (int later = 0;; later++) {
+        HostMech h;
+        read_processes(root, h, instances);
+        if (h.n < 1) throw std::runtime_error("mechanism has no species");
+        h.lanes = lanes > 0 ? lanes : camp_cell_lanes(h.n);
+        if ((h.lanes != 32 && h.lanes != 64 && h.lanes != 128 && h.lanes != 256) || h.n > 8 * h.lanes)
+            throw std::runtime_error("lanes per cell must be 32, 64, 128 or 256, with at most 8 species a lane");
+        build_structure(h);
+        build_tables(h, later);
+        if (!choose_strides(h)) continue;
+        pack_records(h);
+        validate_tables(h);
+        return h;
+    }
 }
 
 AerosolShape aerosol_shape(const char *json, size_t len) {
@@ -1459,8 +1477,27 @@ struct Packer {
 };
 }  // namespace
 
-std::vector<unsigned char> pack_tables(const HostMech &h, DevMech &dm, const unsigned char *base) {
+// The tables that hold storage offsets of the dense block, in one form's storage
+struct FormTables {
+    std::vector<uint32_t> fst, lops;
+    std::vector<int> red, jls, ch;
+    FormTables(const HostMech &h, int f) : fst(h.fst), lops(h.lops), red(h.lred_off), jls(h.jls), ch(h.ch) {
+        for (size_t q = 2; q < jls.size(); q += 4) jls[q] = (jls[q] & ~0xffff) | lu_offset(h, f, jls[q] & 0xffff);
+        for (int &o : red) o = lu_offset(h, f, o);
+        for (size_t q = 0; q < ch.size(); q += 4) ch[q] = lu_offset(h, f, ch[q]);
+        // an op's source is a sparse row's value; its target may be one of the
+        // block, unless it is a partial sum (bit 15 of an update's)
+        for (auto *v : {&fst, &lops})
+            for (uint32_t &op : *v)
+                if ((op & CAMP_OP_DIV) || !(op & 0x8000u))
+                    op = (op & 0xffff0000u) | (uint32_t)lu_offset(h, f, CAMP_OP_TGT(op));
+    }
+};
+
+std::vector<unsigned char> pack_tables(const HostMech &h, DevMech &dm, DevMech &dm64, const unsigned char *base) {
     Packer pk{{}, base};
+    auto int4s = [&](const std::vector<int> &v) { return reinterpret_cast<const int4 *>(pk.put(v)); };
+    const FormTables t4(h, 0);
     dm.n = h.n;
     dm.R = (int)h.procs.size();
     dm.n_env = h.n_env;
@@ -1474,21 +1511,19 @@ std::vector<unsigned char> pack_tables(const HostMech &h, DevMech &dm, const uns
     dm.n_rev = h.n_rev;
     dm.rrev = pk.put(h.rrev);
     dm.nnzJ = (int)h.colidx.size();
-    dm.nlu = h.nlu;
     dm.d = h.d;
     dm.D = h.D;
-    dm.LD = h.LD;
     dm.dbase = h.dbase;
     dm.n_flev = (int)h.flev_ptr.size() - 1;
     dm.fst_ptr = pk.put(h.fst_ptr);
     dm.fst_part = pk.put(h.fst_part);
-    dm.fst = pk.put(h.fst);
-    dm.lops = pk.put(h.lops);
+    dm.fst = pk.put(t4.fst);
+    dm.lops = pk.put(t4.lops);
     dm.lred_ptr = pk.put(h.lred_ptr);
-    dm.lred = reinterpret_cast<const int4 *>(pk.put(h.lred));
-    dm.lred_off = pk.put(h.lred_off);
+    dm.lred = int4s(h.lred);
+    dm.lred_off = pk.put(t4.red);
     dm.ltail = reinterpret_cast<const int2 *>(pk.put(h.ltail));
-    dm.sub_pass = reinterpret_cast<const int4 *>(pk.put(h.sub_pass));
+    dm.sub_pass = int4s(h.sub_pass);
     dm.sub = reinterpret_cast<const int2 *>(pk.put(h.sub));
     dm.n_fpass = h.n_fpass;
     dm.n_bpass = h.n_bpass;
@@ -1498,7 +1533,7 @@ std::vector<unsigned char> pack_tables(const HostMech &h, DevMech &dm, const uns
     dm.n_part = std::max(std::max(h.n_fpart, h.n_spart), h.n_lpart);
     dm.udiag = pk.put(h.udiag);
     dm.perm = pk.put(h.perm);
-    dm.rpack = reinterpret_cast<const int4 *>(pk.put(h.rpack));
+    dm.rpack = int4s(h.rpack);
     dm.gth = reinterpret_cast<const int2 *>(pk.put(h.gth));
     dm.gcf = reinterpret_cast<const double2 *>(pk.put(h.gcf));
     dm.n_gstep = h.n_gstep;
@@ -1508,7 +1543,7 @@ std::vector<unsigned char> pack_tables(const HostMech &h, DevMech &dm, const uns
     dm.n_fpart = h.n_fpart;
     dm.n_fsplit = (int)h.fsplit.size() / 2;
     dm.fsplit = reinterpret_cast<const int2 *>(pk.put(h.fsplit));
-    dm.jls = reinterpret_cast<const int4 *>(pk.put(h.jls));
+    dm.jls = int4s(t4.jls);
     dm.jlc = pk.put(h.jlc);
     std::copy(h.n_jstep, h.n_jstep + 8, dm.n_jstep);
     dm.n_wsec = h.el_phase.empty() ? 0 : h.n_sections;
@@ -1519,19 +1554,31 @@ std::vector<unsigned char> pack_tables(const HostMech &h, DevMech &dm, const uns
     dm.pw_ptr = pk.put(h.pw_ptr);
     dm.pw = pk.put(h.pw);
     dm.n_pp = (int)h.pp.size() / 4;
-    dm.pp = reinterpret_cast<const int4 *>(pk.put(h.pp));
+    dm.pp = int4s(h.pp);
     dm.n_g = h.g_ptr.empty() ? 0 : (int)h.g_ptr.size() - 1;
     dm.g_ptr = pk.put(h.g_ptr);
     dm.g_ent = pk.put(h.g_ent);
     dm.g_coef = pk.put(h.g_coef);
     dm.n_ch = (int)h.ch.size() / 4;
-    dm.ch = reinterpret_cast<const int4 *>(pk.put(h.ch));
+    dm.ch = int4s(t4.ch);
     dm.n_pw = h.n_pw;
     dm.n_pw64 = h.n_pw64;
-    for (int elem : {4, 8})
-        (elem == 4 ? dm.smem4 : dm.smem8) =
-            cell_smem(dm.n, dm.R, dm.n_rev, dm.nlu, elem, dm.n_part, dm.n_fpart, dm.n_pw, dm.n_pw64, dm.lanes);
+    dm.smem4 = form_smem(h, 0, form_nlu(h, h.LD[0]));
+    dm.smem8 = form_smem(h, 1, form_nlu(h, h.LD[1]));
+    dm.LD = h.LD[0];
+    dm.nlu = form_nlu(h, dm.LD);
     bdf_coefficients(dm);
+    dm64 = dm;
+    if (h.LD[1] != h.LD[0]) {
+        const FormTables t8(h, 1);
+        dm64.LD = h.LD[1];
+        dm64.nlu = form_nlu(h, dm64.LD);
+        dm64.fst = pk.put(t8.fst);
+        dm64.lops = pk.put(t8.lops);
+        dm64.lred_off = pk.put(t8.red);
+        dm64.jls = int4s(t8.jls);
+        dm64.ch = int4s(t8.ch);
+    }
     return pk.img;
 }
 

@@ -62,7 +62,8 @@ struct HostMech {
     int n_jstep[8] = {};
     std::vector<int> jptr, jdst, jdiag, jk, jo;
     std::vector<double> jc;
-    int nlu = 0, d = 0, D = 0, LD = 0, dbase = 0;
+    int nlu = 0, d = 0, D = 0, dbase = 0;  // storage with rows of D values in the block
+    int LD[2] = {0, 0};                   // the block's row stride in the FP32 and FP64 forms
     std::vector<int> flev_ptr, frow, fops_ptr;
     std::vector<uint32_t> fops;
     // the factorisation as lane lists (see DevMech)
@@ -121,6 +122,6 @@ void bdf_coefficients(DevMech &dm);
 
 // Pack all device tables into one byte image; `dm` receives offsets
 // relative to `base` (pointers are rebased once the image is on the device).
-std::vector<unsigned char> pack_tables(const HostMech &h, DevMech &dm, const unsigned char *base);
+std::vector<unsigned char> pack_tables(const HostMech &h, DevMech &dm, DevMech &dm64, const unsigned char *base);
 
 }  // namespace camp
