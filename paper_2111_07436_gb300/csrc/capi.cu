@@ -85,7 +85,7 @@ cudaError_t forcing_npl(const DevMech &m, long long n_cells, const double *state
                         double *f, cudaStream_t s) {
     auto kern = campdev::k_forcing<G, NPL, double, W>;
     int smem = camp_cell_smem_bytes(m, 8);
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    cudaError_t e = camp_allow_smem<(W ? 1 << 16 : 0) + G * 16 + NPL>(kern);
     if (e != cudaSuccess) return e;
     kern<<<(unsigned)n_cells, G, smem, s>>>(m, n_cells, state, env, f);
     return cudaGetLastError();
@@ -137,7 +137,7 @@ cudaError_t camp_launch_forcing(const DevMech &m, long long n_cells, const doubl
                                 const double *env, double *f, cudaStream_t s) {
     if (forcing_by_lanes(m, n_cells)) {
         const int rates = 32 * 8 * m.R;
-        cudaError_t e = cudaFuncSetAttribute(campdev::k_forcing_lanes<32>, cudaFuncAttributeMaxDynamicSharedMemorySize, rates);
+        cudaError_t e = camp_allow_smem<0>(campdev::k_forcing_lanes<32>);
         if (e != cudaSuccess) return e;
         campdev::k_forcing_lanes<32><<<(unsigned)((n_cells + 31) / 32), 32, rates, s>>>(m, n_cells, state, env, f);
         return cudaGetLastError();

@@ -4,6 +4,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <atomic>
+
 #include "devmech.h"
 
 #include <nvtx3/nvToolsExt.h>
@@ -18,6 +20,29 @@ struct CampRange {
     CampRange(const CampRange &) = delete;
     CampRange &operator=(const CampRange &) = delete;
 };
+
+// Raise a kernel's dynamic shared-memory limit once to the maximum (the
+// block's 227 KB less the kernel's own static shared memory), so that
+// launches (possibly inside stream capture) make no further attribute calls
+// and no thread lowers the limit between another's call and its launch.
+// One flag per kernel instantiation (the tag) and translation unit, not per
+// function type.  A failed call also clears the runtime's last-error state, so
+// that it is not reported again by a later, healthy launch.
+template <int Tag, class K>
+static cudaError_t camp_allow_smem(K kern) {
+    static std::atomic<int> done_dev{-1};
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess || done_dev == dev) return e;
+    cudaFuncAttributes fa;
+    e = cudaFuncGetAttributes(&fa, kern);
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 227 * 1024 - (int)fa.sharedSizeBytes);
+    if (e == cudaSuccess) done_dev = dev;
+    else (void)cudaGetLastError();
+    return e;
+}
 
 struct SolveArgs {
     long long n_cells;

@@ -16,33 +16,11 @@ namespace {
 using LT = CAMP_LT;
 constexpr bool W = CAMP_WATER != 0;
 
-// Raise a kernel's dynamic shared-memory limit once to the maximum (the
-// block's 227 KB less the kernel's own static shared memory), so that
-// launches (possibly inside stream capture) make no further attribute calls.
-// One flag per kernel instantiation (the tag), not per function type.  A
-// failed call also clears the runtime's last-error state, so that it is not
-// reported again by a later, healthy launch.
-template <int Tag, class K>
-cudaError_t allow_smem(K kern) {
-    static int done_dev = -1;
-    int dev = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e != cudaSuccess || done_dev == dev) return e;
-    cudaFuncAttributes fa;
-    e = cudaFuncGetAttributes(&fa, kern);
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 227 * 1024 - (int)fa.sharedSizeBytes);
-    if (e == cudaSuccess) done_dev = dev;
-    else (void)cudaGetLastError();
-    return e;
-}
-
 template <int G, int NPL>
 cudaError_t launch_solve_npl(const DevMech &m, const SolveArgs &a, int grid, cudaStream_t s) {
     auto kern = campdev::k_solve<G, NPL, LT, W>;
     int smem = camp_cell_smem_bytes(m, (int)sizeof(LT)) * a.cpb;
-    cudaError_t e = allow_smem<G * 16 + NPL>(kern);
+    cudaError_t e = camp_allow_smem<G * 16 + NPL>(kern);
     if (e != cudaSuccess) return e;
     kern<<<grid, G * a.cpb, smem, s>>>(m, a);
     return cudaGetLastError();
@@ -52,7 +30,7 @@ template <int G, int NPL>
 cudaError_t occupancy_npl(const DevMech &m, int cpb, int *blocks) {
     auto kern = campdev::k_solve<G, NPL, LT, W>;
     int smem = camp_cell_smem_bytes(m, (int)sizeof(LT)) * cpb;
-    cudaError_t e = allow_smem<G * 16 + NPL>(kern);
+    cudaError_t e = camp_allow_smem<G * 16 + NPL>(kern);
     if (e != cudaSuccess) return e;
     return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks, kern, G * cpb, smem);
 }
@@ -62,7 +40,7 @@ cudaError_t launch_jac_npl(const DevMech &m, long long n_cells, const double *st
                            const double *env, double *jac, cudaStream_t s) {
     auto kern = campdev::k_jacobian<G, NPL, LT, W>;
     int smem = camp_cell_smem_bytes(m, (int)sizeof(LT));
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    cudaError_t e = camp_allow_smem<G * 16 + NPL>(kern);
     if (e != cudaSuccess) return e;
     kern<<<(unsigned)n_cells, G, smem, s>>>(m, n_cells, state, env, jac);
     return cudaGetLastError();
@@ -74,7 +52,7 @@ cudaError_t launch_lu_npl(const DevMech &m, long long n_cells, const double *sta
                           cudaStream_t s) {
     auto kern = campdev::k_lu_solve<G, NPL, LT, W>;
     int smem = camp_cell_smem_bytes(m, (int)sizeof(LT));
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    cudaError_t e = camp_allow_smem<G * 16 + NPL>(kern);
     if (e != cudaSuccess) return e;
     kern<<<(unsigned)n_cells, G, smem, s>>>(m, n_cells, state, env, gamma, b, x, status);
     return cudaGetLastError();
