@@ -119,23 +119,36 @@ cudaError_t camp_launch_rates(const DevMech &m, long long n_cells, const double 
     return cudaGetLastError();
 }
 
-// Whether f takes a lane a cell (k_forcing_lanes).  A warp of 32 cells takes
-// the same time however many there are, up to four warps an SM (19456
-// cells): 0.82 ms for the 72-species mechanism (186 processes), 0.056 ms for
-// 12 processes.  A warp a cell, R / 32 processes at a time, takes 0.82 ms for
-// 13000 cells of the former and 0.056 ms for 1500 of the latter (3.45 ms
-// against 5.83 ms for 65537 gas-72 cells, 0.12 against 2.2 ms of the small
-// mechanism's, before the exact powers were skipped).  One-warp cells without
-// a water parameter only: their sums are not split, so both kernels add them
-// in the same order; four warps' rates have to fit an SM.
-static bool forcing_by_lanes(const DevMech &m, long long n_cells) {
-    return m.lanes == 32 && m.n_wsec == 0 && 4 * (32 * 8 * m.R + 1024) <= 228 * 1024 &&
-           n_cells * ((m.R + 31) / 32 * 32) >= 13000LL * m.R;
+// Whether f of n_cells cells is faster with a lane a cell (k_forcing_lanes)
+// than with a warp a cell, from the times of both on 256 to 65536 cells of
+// mechanisms of 12 to 222 processes.  A lane a cell: 4.3 us a process for up to
+// 2 warps of 32 cells an SM, 0.5 + 0.18 k times that for k warps together, and
+// as many of them as their rates leave room for (186 processes: 4, so that
+// 19457 cells start a second wave: 0.90 -> 1.61 ms).  A warp a cell: 1.63 us a
+// cell and SM for every 32 processes, and at least 2.4 us and 1.14 us for each
+// 32 (more where exp and pow are spread over the processes).  The line: 12
+// processes at 2200 cells (measured 1500), 61 at 8500 (9300), 186 at 12400 up
+// to 19456, at 27600 up to 38912 and at 42800 (13300, 29200, 43000).
+// Exported for the tests.
+extern "C" int camp_forcing_by_lanes(int processes, long long n_cells, int sm_count) {
+    const int R = processes, by32 = (R + 31) / 32, room = std::min(32, 228 * 1024 / (32 * 8 * R + 1024));
+    if (room < 4) return 0;
+    auto together = [](double k) { return std::max(1.0, 0.5 + 0.18 * k); };
+    const long long warps = (n_cells + 31) / 32, wave = (long long)room * sm_count, rest = warps % wave;
+    const double lanes = 4.3 * R * ((double)(warps / wave) * together(room) +
+                                    (rest ? together((double)rest / sm_count) : 0.0));
+    return lanes < std::max(1.63 * by32, 2.4 + 1.14 * by32) * (double)n_cells / sm_count;
 }
 
-cudaError_t camp_launch_forcing(const DevMech &m, long long n_cells, const double *state,
-                                const double *env, double *f, cudaStream_t s) {
-    if (forcing_by_lanes(m, n_cells)) {
+// One-warp cells without a water parameter only: their sums are not split, so
+// both kernels add them in the same order.
+static bool forcing_by_lanes(const DevMech &m, long long n_cells, int sm_count) {
+    return m.lanes == 32 && m.n_wsec == 0 && camp_forcing_by_lanes(m.R, n_cells, sm_count);
+}
+
+cudaError_t camp_launch_forcing(const DevMech &m, long long n_cells, const double *state, const double *env, double *f,
+                                int sm_count, cudaStream_t s) {
+    if (forcing_by_lanes(m, n_cells, sm_count)) {
         const int rates = 32 * 8 * m.R;
         cudaError_t e = camp_allow_smem<0>(campdev::k_forcing_lanes<32>);
         if (e != cudaSuccess) return e;
@@ -907,7 +920,7 @@ int camp_forcing(const camp_mech *m, int64_t n_cells, const double *state, const
         CUDA_TRY(camp_arrow_forcing(m->dm, m->ad, n_cells, state, env, f, (cudaStream_t)stream));
         return CAMP_OK;
     }
-    CUDA_TRY(camp_launch_forcing(m->dm64, n_cells, state, env, f, (cudaStream_t)stream));
+    CUDA_TRY(camp_launch_forcing(m->dm64, n_cells, state, env, f, m->sm_count, (cudaStream_t)stream));
     return CAMP_OK;
 }
 

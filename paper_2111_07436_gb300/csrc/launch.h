@@ -100,8 +100,8 @@ cudaError_t camp_launch_lu_solve_f64w(const DevMech &m, long long n_cells, const
 
 cudaError_t camp_launch_rates(const DevMech &m, long long n_cells, const double *env, double *kf,
                               double *kr, cudaStream_t s);
-cudaError_t camp_launch_forcing(const DevMech &m, long long n_cells, const double *state,
-                                const double *env, double *f, cudaStream_t s);
+cudaError_t camp_launch_forcing(const DevMech &m, long long n_cells, const double *state, const double *env, double *f,
+                                int sm_count, cudaStream_t s);
 cudaError_t camp_launch_jacobian_f32(const DevMech &m, long long n_cells, const double *state,
                                      const double *env, double *jac, cudaStream_t s);
 cudaError_t camp_launch_jacobian_f64(const DevMech &m, long long n_cells, const double *state,
