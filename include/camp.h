@@ -189,8 +189,8 @@ typedef struct {
     int32_t max_steps;       /* internal steps per cell (default 10000) */
     int32_t cells_per_block; /* 0: the autotuned choice if any, else the
                                 count (1..4) with the most resident cells
-                                (1 when all cells are resident at one a
-                                block).
+                                (1 when all cells, a batch's other groups
+                                included, are resident at one a block).
                                 Block-arrow (particle-resolved) mechanisms:
                                 CTAs per cluster, 1, 2, 4, 8 or 16 (0: 8) */
     double hmin_frac;        /* minimum step = hmin_frac * dt (default 1e-10) */

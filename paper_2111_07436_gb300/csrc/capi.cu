@@ -502,9 +502,52 @@ static int arrow_solve(camp_mech *m, int64_t n_cells, double *state, const doubl
     return CAMP_OK;
 }
 
+// Blocks of cpb cells that an SM holds (asked once per mechanism)
+static cudaError_t solve_occupancy(camp_mech *m, int variant, int cpb, int *per_sm) {
+    int &known = m->occ[variant][cpb];
+    if (known == 0) {
+        const bool w = m->dm.n_wsec > 0;
+        cudaError_t e = variant == CAMP_VARIANT_MIXED
+                            ? (w ? camp_occupancy_f32w(m->dm, cpb, per_sm) : camp_occupancy_f32(m->dm, cpb, per_sm))
+                            : (w ? camp_occupancy_f64w(m->dm64, cpb, per_sm) : camp_occupancy_f64(m->dm64, cpb, per_sm));
+        if (e != cudaSuccess) return e;
+        known = *per_sm > 0 ? *per_sm : -1;
+    }
+    *per_sm = known > 0 ? known : 0;
+    return cudaSuccess;
+}
+
+// Share of the device that a solve takes at one cell a block (1: all of it)
+static double device_share(const camp_mech *mc, int64_t n_cells, int variant) {
+    camp_mech *m = const_cast<camp_mech *>(mc);
+    if (m->arrow || !m->on_device || (variant != CAMP_VARIANT_MIXED && variant != CAMP_VARIANT_FP64)) return 1.0;
+    int one = 0;
+    if (solve_occupancy(m, variant, 1, &one) != cudaSuccess || one < 1) return 1.0;
+    return (double)n_cells / ((double)one * m->sm_count);
+}
+
+// Cells a block takes by default: as many as give the most resident cells
+// (blocks_per_sm[c]: blocks of c cells an SM holds, c up to most), the fewest
+// on ties.  Cells that are all resident at one a block spread evenly over the
+// SMs that way (256 gas-72 cells: 6.6 ms, 6.9 ms at three a block), but only if
+// the rest of the device is free: `beside` is the share of it that the other
+// groups of a batch take (8 groups of 256 cells: 13.6 ms at one a block, 12.8
+// at three).  The chunks of the serving loop start and end one by one and are
+// as fast either way (256 cells: 40.0 and 39.4 ms for 32 of them; 1024 cells:
+// 62.3 and 63.5 ms for 16).  Exported for the tests.
+extern "C" int camp_default_cells_per_block(const int *blocks_per_sm, int most, long long n_cells, int sm_count,
+                                            double beside) {
+    const double room = (double)blocks_per_sm[1] * sm_count;
+    if ((double)n_cells + beside * room <= room) return 1;
+    int best = 0, cpb = 1;
+    for (int c = 1; c <= most; c++)
+        if (blocks_per_sm[c] * c > best) { best = blocks_per_sm[c] * c; cpb = c; }
+    return cpb;
+}
+
 static int solve_impl(const camp_mech *mc, int64_t n_cells, double *state, const double *env, double dt,
                       int32_t n_outer, double *traj, double rtol, const double *atol, int32_t atol_len,
-                      int32_t *status, const camp_solve_opts *opts, void *stream) {
+                      int32_t *status, const camp_solve_opts *opts, void *stream, double beside = 0.0) {
     camp_mech *m = const_cast<camp_mech *>(mc);
     if (n_outer < 1) return fail(CAMP_E_INVAL, "n_steps must be at least 1");
     if (!m) return fail(CAMP_E_INVAL, "NULL mechanism");
@@ -530,33 +573,14 @@ static int solve_impl(const camp_mech *mc, int64_t n_cells, double *state, const
     if (o.persistent < 0)
         o.persistent = m->tuned_persistent[o.variant] >= 0 ? m->tuned_persistent[o.variant]
                                                            : (o.variant == CAMP_VARIANT_MIXED ? 1 : 0);
-    auto occupancy = [&](int cpb_, int *per_sm) -> cudaError_t {
-        if (m->occ[o.variant][cpb_] == 0) {
-            const bool w = m->dm.n_wsec > 0;
-            cudaError_t e = f32 ? (w ? camp_occupancy_f32w(m->dm, cpb_, per_sm) : camp_occupancy_f32(m->dm, cpb_, per_sm))
-                                : (w ? camp_occupancy_f64w(m->dm64, cpb_, per_sm) : camp_occupancy_f64(m->dm64, cpb_, per_sm));
-            if (e != cudaSuccess) return e;
-            m->occ[o.variant][cpb_] = *per_sm > 0 ? *per_sm : -1;
-        }
-        *per_sm = m->occ[o.variant][cpb_] > 0 ? m->occ[o.variant][cpb_] : 0;
-        return cudaSuccess;
-    };
     int cpb = o.cells_per_block > 0 ? o.cells_per_block : m->tuned_cpb[o.variant];
-    if (cpb <= 0) {  // most resident cells per SM, fewest cells per block on ties
-        int best = 0;
-        cpb = 1;
-        int max_cpb = m->h.lanes > 32 ? 1 : 4;
-        // a call whose cells are all resident at one a block spreads evenly
-        // over the SMs that way (256 gas cells: 6.3 ms; 7.3 ms at three a block)
-        int one = 0;
-        CUDA_TRY(occupancy(1, &one));
-        if (n_cells <= (long long)one * m->sm_count) max_cpb = 1;
-        for (int c2 = 1; c2 <= max_cpb; c2++) {
-            if (c2 * smem_cell > kMaxSmem) break;
-            int per_sm = 0;
-            CUDA_TRY(occupancy(c2, &per_sm));
-            if (per_sm * c2 > best) { best = per_sm * c2; cpb = c2; }
+    if (cpb <= 0) {
+        int per_sm[5] = {}, most = 0;
+        while (most < (m->h.lanes > 32 ? 1 : 4) && (most + 1) * smem_cell <= kMaxSmem) {
+            most++;
+            CUDA_TRY(solve_occupancy(m, o.variant, most, &per_sm[most]));
         }
+        cpb = camp_default_cells_per_block(per_sm, most, n_cells, m->sm_count, beside);
     }
     cpb = std::min(cpb, 4);
     while (cpb > 1 && cpb * smem_cell > kMaxSmem) cpb--;
@@ -592,7 +616,7 @@ static int solve_impl(const camp_mech *mc, int64_t n_cells, double *state, const
             q = m->own_ws;
         }
         int per_sm = 0;
-        CUDA_TRY(occupancy(cpb, &per_sm));
+        CUDA_TRY(solve_occupancy(m, o.variant, cpb, &per_sm));
         if (per_sm < 1) return fail(CAMP_E_UNSUPPORTED, "kernel does not fit on an SM");
         grid = std::min<long long>((long long)per_sm * m->sm_count, (n_cells + cpb - 1) / cpb);
         CUDA_TRY(cudaMemsetAsync(q, 0, sizeof(unsigned long long), s));
@@ -688,7 +712,8 @@ int camp_solve_batch(const camp_group *groups, int32_t n_groups, double dt, doub
     // until its counter runs dry, so the groups run one after the other and
     // the last group's cells make the batch's tail -- best the shortest ones
     int order[CAMP_MAX_GROUPS];
-    double work[CAMP_MAX_GROUPS];
+    double work[CAMP_MAX_GROUPS], share[CAMP_MAX_GROUPS], total = 0.0;
+    const int variant = opts ? opts->variant : CAMP_VARIANT_MIXED;
     for (int g = 0; g < n_groups; g++) {
         if (!groups[g].mech) return fail(CAMP_E_INVAL, "NULL mechanism in group");
         const camp::HostMech &h = groups[g].mech->h;
@@ -697,6 +722,8 @@ int camp_solve_batch(const camp_group *groups, int32_t n_groups, double dt, doub
                                  20LL * groups[g].mech->n)
                       : (double)(h.flops_forcing + h.flops_solve + 20 * h.n);
         order[g] = g;
+        share[g] = n_groups > 1 ? device_share(groups[g].mech, groups[g].n_cells, variant) : 0.0;
+        total += share[g];
     }
     std::sort(order, order + n_groups, [&](int a, int b) { return work[a] > work[b]; });
     cudaStream_t parent = (cudaStream_t)stream;
@@ -727,8 +754,8 @@ int camp_solve_batch(const camp_group *groups, int32_t n_groups, double dt, doub
         if (o.persistent < 0) o.persistent = 1;
         if (!o.workspace && n_groups > 1 && o.persistent)
             return fail(CAMP_E_INVAL, "each group of a multi-group persistent solve needs its own workspace");
-        rc = camp_solve(gr.mech, gr.n_cells, gr.state, gr.env, dt, rtol, gr.atol, gr.atol_len, gr.status,
-                        &o, forks[i]);
+        rc = solve_impl(gr.mech, gr.n_cells, gr.state, gr.env, dt, 1, nullptr, rtol, gr.atol, gr.atol_len, gr.status,
+                        &o, forks[i], total - share[order[i]]);
         CUDA_TRY(cudaEventRecord(ev_join[i], forks[i]));
         CUDA_TRY(cudaStreamWaitEvent(parent, ev_join[i], 0));
         if (rc != CAMP_OK) return rc;
