@@ -34,8 +34,12 @@ namespace cg = cooperative_groups;
 constexpr int ARROW_NT = 256;     // threads per CTA
 // CTAs an SM holds.  The particle loops are chains of loads and of FP64
 // instructions that one warp issues every 64 cycles, so warps count for more
-// than registers (10^4 particles, 152 cells, mixed / FP64 form: 2 CTAs 183 /
-// 236 ms, 3: 148 / 192, 4: 134 / 180, 5: 125 / 173, 6: 132 / 184).
+// than registers (10^4 particles of 7 species, 152 cells, 180 s, mixed / FP64
+// form: 2 CTAs 183 / 236 ms, 3: 148 / 192, 4: 134 / 180, 5: 125 / 173, 6: 132 /
+// 184).  More than 8 species a particle spill 2.7 / 4.0 KB at 5 CTAs and are
+// faster all the same than runtime loops at 4 (152 cells, 60 s: 9 species 31.7
+// -> 27.4 / 40.2 -> 39.0 ms, 12: 44.1 -> 37.1 / 56.3 -> 51.0, 16: 62.7 -> 52.3 /
+// 81.7 -> 69.6); other counts were not timed for them.
 constexpr int ARROW_CTAS = 5;
 constexpr int ARROW_MAX_CL = 16;  // CTAs per cluster
 constexpr int ARROW_MAX_RG = 64;  // gas processes

@@ -117,8 +117,6 @@ __device__ __forceinline__ double ipowd(double x, int k) {
     return r;
 }
 
-// A exp(C/T) (T/300)^B: the Arrhenius terms of the Troe and custom rate
-// constants (D = 300 K, E = 0)
 // exp(c / T) and (T / d)^b.  With c = 0 or b = 0 (most mechanisms' case) they
 // are exactly 1 for a positive T, without the ~20 and ~80 FP64 instructions,
 // each a warp's for 64 cycles, of the functions.
@@ -128,6 +126,8 @@ __device__ __forceinline__ double exp_over(double c, double T) {
 __device__ __forceinline__ double pow_over(double T, double d, double b) {
     return b == 0.0 ? 1.0 : pow(T / d, b);
 }
+// A exp(C/T) (T/300)^B: the Arrhenius terms of the Troe and custom rate
+// constants (D = 300 K, E = 0)
 __device__ __forceinline__ double arr300(const double *par, double T) {
     return __ldg(par) * exp_over(__ldg(par + 2), T) * pow_over(T, 300.0, __ldg(par + 1));
 }
@@ -1490,8 +1490,10 @@ __device__ int integrate_cell(const DevMech &m, const CellPtr<LT> &c, double *__
     const int n = m.n;
     constexpr bool EXACT = sizeof(LT) == 8;  // the plain FP64 form
     // whether z1 / l1 is rounded before the Newton residual takes it or fused
-    // into its sum: fixed per shape, so that a build's choice of contractions
-    // cannot move a cell's step sequence
+    // into its sum.  Either form would do in every shape; the condition
+    // reproduces what the compiler chose for each before it was written out, so
+    // that results stay the same, now whatever a build contracts.  (A cell thus
+    // takes one or the other with its shape, as it takes other orders of sums.)
     constexpr bool ROUND_Z1 = G == 32 && !W && (EXACT || NPL <= 3);
     using C = Ctl<EXACT>;
     const double h_in = step_io ? *step_io : 0.0;

@@ -154,7 +154,8 @@ __global__ void k_forcing(const __grid_constant__ DevMech m, long long n_cells, 
 // cells lie in shared memory ([process][cell]); the state and env rows are
 // read in place (each lane its own row: the loads are few beside the FP64
 // work).  The sums take their entries in the order, and in the two
-// accumulators, of the cell kernels: the same f bit for bit.
+// accumulators, of the cell kernels: the same f bit for bit.  (L is always 32;
+// as a template the kernel may stand in a header of several units.)
 template <int L>
 __global__ void __launch_bounds__(L) k_forcing_lanes(const __grid_constant__ DevMech m, long long n_cells,
                                                       const double *state, const double *env, double *f_out) {

@@ -8,8 +8,9 @@ namespace campdev {
 // Every cell over one or more outer steps; clusters take cells round-robin
 // (cluster c: cells c, c + clusters, ...), each with its own slice of the
 // scratch.  NPM: the compiler's bound of the phase species per particle (8 up
-// to 8 species, else 16; with runtime loops instead the kernel took 148.5
-// against 124.9 ms on 152 cells of 10^4 particles, 7 species each).
+// to 8 species, else 16; with runtime loops, at four CTAs an SM, the kernel
+// took 149.7 ms instead of 124.2 on 152 cells of 10^4 particles of 7 species,
+// 188.6 instead of 172.3 in the FP64 form).
 template <typename LT, int NPM>
 __global__ void __launch_bounds__(ARROW_NT, ARROW_CTAS)
     k_arrow(const __grid_constant__ DevMech mt, const __grid_constant__ ArrowDev a, const __grid_constant__ SolveArgs s,
