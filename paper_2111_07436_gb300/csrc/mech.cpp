@@ -834,7 +834,7 @@ static void build_tables(HostMech &h, int later) {
     h.D = n - h.d;
 
     // storage offsets: sparse rows < d, the L21 part of rows >= d, then the
-    // block with rows of D values (lu_offset gives a form's own)
+    // block with rows of D values (lu_offsets gives a form's own)
     std::vector<int> lu_off(h.lu_colidx.size(), -1);
     int nsp = 0;
     for (int i = 0; i < n; i++)
@@ -1139,10 +1139,12 @@ static void build_tables(HostMech &h, int later) {
     h.sub_pass.insert(h.sub_pass.end(), 4 * (size_t)h.lanes, -1);
 }
 
-// Storage offset of a table entry in the FP32 (f = 0) or FP64 (1) form
-static int lu_offset(const HostMech &h, int f, int o) {
-    const int q = o - h.dbase;
-    return h.D == 0 || q < 0 ? o : h.dbase + q / h.D * h.LD[f] + q % h.D;
+// Storage offsets of the tables' entries in the FP32 (f = 0) or FP64 (1) form
+static std::vector<int> lu_offsets(const HostMech &h, int f) {
+    std::vector<int> to(h.nlu);
+    for (int o = 0; o < h.dbase; o++) to[o] = o;
+    for (int o = h.dbase; o < h.nlu; o++) to[o] = h.dbase + (o - h.dbase) / h.D * h.LD[f] + (o - h.dbase) % h.D;
+    return to;
 }
 static int form_nlu(const HostMech &h, int stride) { return h.dbase + h.D * stride; }
 static CellSmem form_smem(const HostMech &h, int f, int nlu) {
@@ -1482,15 +1484,15 @@ struct FormTables {
     std::vector<uint32_t> fst, lops;
     std::vector<int> red, jls, ch;
     FormTables(const HostMech &h, int f) : fst(h.fst), lops(h.lops), red(h.lred_off), jls(h.jls), ch(h.ch) {
-        for (size_t q = 2; q < jls.size(); q += 4) jls[q] = (jls[q] & ~0xffff) | lu_offset(h, f, jls[q] & 0xffff);
-        for (int &o : red) o = lu_offset(h, f, o);
-        for (size_t q = 0; q < ch.size(); q += 4) ch[q] = lu_offset(h, f, ch[q]);
+        const std::vector<int> to = lu_offsets(h, f);
+        for (size_t q = 2; q < jls.size(); q += 4) jls[q] = (jls[q] & ~0xffff) | to[jls[q] & 0xffff];
+        for (int &o : red) o = to[o];
+        for (size_t q = 0; q < ch.size(); q += 4) ch[q] = to[ch[q]];
         // an op's source is a sparse row's value; its target may be one of the
         // block, unless it is a partial sum (bit 15 of an update's)
         for (auto *v : {&fst, &lops})
             for (uint32_t &op : *v)
-                if ((op & CAMP_OP_DIV) || !(op & 0x8000u))
-                    op = (op & 0xffff0000u) | (uint32_t)lu_offset(h, f, CAMP_OP_TGT(op));
+                if ((op & CAMP_OP_DIV) || !(op & 0x8000u)) op = (op & 0xffff0000u) | (uint32_t)to[CAMP_OP_TGT(op)];
     }
 };
 
