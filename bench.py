@@ -49,12 +49,12 @@ HBM_FALLBACK_GBS = 6800.0          # used only when the measured peaks file is a
 # particles10k: 19), scaled by the cells of the timed launch.  Valid only for the kernel sources whose digest
 # is given: the bench reports null traffic once the kernels have changed.
 DRAM_BYTES_PER_CELL = {
-    "uneven": {"digest": "7ad162b3d2e196cb", "bytes_per_cell": [14963200 / 14734, 4632832 / 1650]},
-    "gas72": {"digest": "7ad162b3d2e196cb", "bytes_per_cell": [4560384 / 4096]},
-    "multiphase232": {"digest": "7ad162b3d2e196cb", "bytes_per_cell": [5745152 / 2048]},
-    "particles": {"digest": "7ad162b3d2e196cb", "bytes_per_cell": [6214144 / 512]},
-    "water": {"digest": "7ad162b3d2e196cb", "bytes_per_cell": [5969408 / 2048]},
-    "particles10k": {"digest": "9df31e777d01acd0", "bytes_per_cell": [(11711516416 + 6147372544) / 19]},
+    "uneven": {"digest": "000c924887f84e5d", "bytes_per_cell": [(15158528 + 192000) / 14734, (5056000 + 71168) / 1650]},
+    "gas72": {"digest": "000c924887f84e5d", "bytes_per_cell": [(4716800 + 54016) / 4096]},
+    "multiphase232": {"digest": "000c924887f84e5d", "bytes_per_cell": [(5547264 + 59392) / 2048]},
+    "particles": {"digest": "000c924887f84e5d", "bytes_per_cell": [(6164736 + 25856) / 512]},
+    "water": {"digest": "000c924887f84e5d", "bytes_per_cell": [(6053120 + 55552) / 2048]},
+    "particles10k": {"digest": "a96f2ba6108b3899", "bytes_per_cell": [(12244228352 + 6729125632) / 19]},
 }
 
 
